@@ -286,7 +286,8 @@ int lbm_probe(lbm_handle h, int n, const int64_t *cells, double *p_prime);
  * lbm_set_launch -- launch shape of the update kernel (a tuning knob; the
  * result does not depend on it beyond FP round-off order).
  *   block            : threads per block, a multiple of 32 in [32, 256], or 0
- *                      for the default (128 one cell per thread, else 64)
+ *                      for the default (128 one cell per thread, else the multiple
+ *                      of 32 up to 96 that leaves no idle warp in a row)
  *   cells_per_thread : 1 = one cell per thread (the general kernel); 2 or 4 =
  *                      vectorised kernel with that many consecutive x cells per
  *                      thread (FP64: 2; FP32, FP16, BF16: 2 or 4); 0 = default

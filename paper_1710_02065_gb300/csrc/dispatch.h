@@ -65,7 +65,20 @@ inline int vec_default(int lattice, int precision)
     if (precision == PREC_FP32) return lattice == 2 /* D3Q27 */ ? 2 : 1;
     return 2;
 }
-inline int block_default(int vec) { return vec == 1 ? 128 : 64; }
+// Default threads per block.  The vectorised kernel's blocks lie along x
+// rows of nx / vec threads, so the block has to divide the row's warps or the
+// last block of every row holds idle warps: 64 threads where the row is a
+// whole number of 64-thread blocks, one block for a row of up to three warps,
+// else single warps.  Measured on GB300 (16-bit storage, two cells per
+// thread), us per step at 64 / 32 / 96 threads: rows of 96 threads (192 x 128 x
+// 128 jet) D3Q27 96.8 / 78.2 / 76.0, D3Q19 63.9 / 50.6 / 51.5; rows of 192 threads
+// (384 x 256 x 256 jet) D3Q19 338.6 / 336.8 / 338.6.
+inline int block_default(int vec, int nx)
+{
+    if (vec == 1) return 128;
+    const int row = (nx / vec + 31) / 32 * 32;
+    return row % 64 == 0 ? 64 : (row <= 96 ? row : 32);
+}
 
 // Row-staged kernel (bulk copies of whole rows into shared memory; FP32,
 // FP16, BF16; no cell-type mask; nx * element size a multiple of 16 bytes).

@@ -1089,7 +1089,7 @@ static cudaError_t launch_update(lbm_ctx *h, const StepParams &p, const void *fi
     if (p.bgk) {
         // plain BGK: the general kernel only
         h->launches += 1;
-        return step_general(h, p, fin, fout, h->block > 0 ? h->block : block_default(1));
+        return step_general(h, p, fin, fout, h->block > 0 ? h->block : block_default(1, p.n[0]));
     }
     if (staging_wanted(h) && h->lattice != LBM_D3Q27) {
         const cudaError_t e = h->lattice == LBM_D2Q9
@@ -1104,7 +1104,7 @@ static cudaError_t launch_update(lbm_ctx *h, const StepParams &p, const void *fi
     }
     int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
     if (!vec_eligible(p) || vec == 1 || !vec_available(h, vec) || p.n[0] % vec != 0) vec = 1;
-    const int block = h->block > 0 ? h->block : block_default(vec);
+    const int block = h->block > 0 ? h->block : block_default(vec, p.n[0]);
     h->launches += 1;
     if (vec == 1) return step_general(h, p, fin, fout, block);
     switch (h->lattice) {
@@ -1266,7 +1266,7 @@ static cudaError_t aa_step(lbm_ctx *h, const StepParams &p)
     const bool loc = h->aa_odd != 0;
     int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
     if (!vec_eligible(p) || vec == 1 || !vec_available(h, vec) || p.n[0] % vec != 0) vec = 1;
-    const int block = h->block > 0 ? h->block : block_default(vec);
+    const int block = h->block > 0 ? h->block : block_default(vec, p.n[0]);
     h->launches += 1;
     h->aa_odd ^= 1;
     if (vec > 1) {
@@ -1726,7 +1726,7 @@ extern "C" int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread)
     CHECK_HANDLE(h);
     int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
     if (h->solid_d || vec == 1 || !vec_available(h, vec) || h->n[0] % vec != 0) vec = 1;
-    if (block) *block = h->block > 0 ? h->block : block_default(vec);  // level 0
+    if (block) *block = h->block > 0 ? h->block : block_default(vec, h->n[0]);  // level 0
     if (cells_per_thread) *cells_per_thread = vec;
     return LBM_OK;
 }
