@@ -1186,10 +1186,11 @@ static cudaError_t refine_kernels3(lbm_ctx *h, int k, int stage, int a_half)
     return cudaGetLastError();
 }
 
-// Coupling of refined level k >= 1 with its parent k - 1:
+// Coupling of refined level k >= 1 with its parent k - 1 (2D: stage 3 only, the
+// rest runs inside the level's own substeps, launch_level_2d):
 //   stage 0: parent-side interface moments at t + 1 from the pre-step parent field
-//   stage 1: level k's ring / shell at t + 1/2 (a_half = 1) or t + 1 (a_half = 0)
-//   stage 2: the parent's covered ring / shell from level k at t + 1/2
+//   stage 1: level k's shell at t + 1/2 (a_half = 1) or t + 1 (a_half = 0)
+//   stage 2: the parent's covered shell from level k at t + 1/2
 //   stage 3: interface moments at t = 0 (local moments of the stored parent field)
 template <class S>
 static cudaError_t refine_kernels(lbm_ctx *h, int k, int stage, int a_half)
@@ -1198,37 +1199,8 @@ static cudaError_t refine_kernels(lbm_ctx *h, int k, int stage, int a_half)
     if (h->d == 3) return refine_kernels3<D3Q19, S>(h, k, stage, a_half);
     FineLevel *F = fine_level(h, k);
     const GridRef P = level_grid(h, k - 1);
-    const double tau_p = level_tau(h, k - 1);
-    const RefineGeom &g = F->geom;
-    cudaStream_t st = h->stream;
-    switch (stage) {
-    case 0: {  // coarse line moments at t + 1 from the pre-step coarse field
-        const int n = line_count(g);
-        k_line_moments<S><<<grid1(n, 128), 128, 0, st>>>(g, (const S *)P.f[*P.cur], links_mask(h, k - 1), 1,
-                                                          (CT<S> *)F->M[1 - F->mcur]);
-        break;
-    }
-    case 1: {  // fine ring at t + 1/2 (a_half = 1) or t + 1 (a_half = 0)
-        const int n = 2 * g.nfx + 2 * (g.nfy - 2);
-        k_fill_ring<S><<<grid1(n, 128), 128, 0, st>>>(
-            g, (const CT<S> *)F->M[F->mcur], (const CT<S> *)F->M[1 - F->mcur], CT<S>(a_half ? 0.5 : 1.0),
-            CT<S>(F->tau / (2.0 * tau_p)), CT<S>(1.0 - 1.0 / F->tau), (S *)F->f[F->cur]);
-        break;
-    }
-    case 2: {  // covered coarse ring from the fine field; pre-collision fine moments pulled from f(t + 1/2)
-        const int n = 2 * (g.Wc - 1) + 2 * (g.Hc - 3);
-        k_restrict<S><<<grid1(n, 128), 128, 0, st>>>(g, (const S *)F->f[1 - F->cur], links_mask(h, k),
-                                                      CT<S>(2.0 * tau_p / F->tau), CT<S>(1.0 - 1.0 / tau_p),
-                                                      (S *)P.f[*P.cur]);
-        break;
-    }
-    case 3: {  // line moments at t = 0: local moments of the stored coarse field
-        const int n = line_count(g);
-        k_line_moments<S><<<grid1(n, 128), 128, 0, st>>>(g, (const S *)P.f[*P.cur], links_mask(h, k - 1), 0,
-                                                          (CT<S> *)F->M[F->mcur]);
-        break;
-    }
-    }
+    const int n = line_count(F->geom);
+    k_line_moments<S><<<grid1(n, 128), 128, 0, h->stream>>>(F->geom, (const S *)P.f[*P.cur], (CT<S> *)F->M[F->mcur]);
     h->launches += 1;
     return cudaGetLastError();
 }
@@ -1240,6 +1212,40 @@ static cudaError_t refine_stage(lbm_ctx *h, int k, int stage, int a_half = 0)
     case LBM_FP32: return refine_kernels<float>(h, k, stage, a_half);
     case LBM_FP16_SHIFTED: return refine_kernels<__half>(h, k, stage, a_half);
     case LBM_BF16_SHIFTED: return refine_kernels<__nv_bfloat16>(h, k, stage, a_half);
+    }
+    return cudaErrorInvalidValue;
+}
+
+// Substep `sub` (0, 1) of refined 2D level k >= 1 with its coupling.  The
+// parent's update has been launched already: its lattice *P.cur is the field
+// at t + 1, the other one the pre-step field.
+static cudaError_t launch_level_2d(lbm_ctx *h, const StepParams &p, int k, int sub)
+{
+    FineLevel *F = fine_level(h, k);
+    const GridRef P = level_grid(h, k - 1);
+    const double tau_p = level_tau(h, k - 1);
+    LevelStep2D q{};
+    q.g = F->geom;
+    q.parent_old = P.f[1 - *P.cur];
+    q.parent_new = P.f[*P.cur];
+    q.parent_links = links_mask(h, k - 1);
+    q.level_links = links_mask(h, k);
+    q.M0 = F->M[F->mcur];
+    q.M1 = F->M[1 - F->mcur];
+    q.first = sub == 0 ? 1 : 0;
+    q.a = sub == 0 ? 0.5 : 1.0;
+    q.alpha_down = F->tau / (2.0 * tau_p);
+    q.omega_down = 1.0 - 1.0 / F->tau;
+    q.alpha_up = 2.0 * tau_p / F->tau;
+    q.omega_up = 1.0 - 1.0 / tau_p;
+    const void *fin = F->f[F->cur];
+    void *fout = F->f[1 - F->cur];
+    h->launches += 1;
+    switch (h->prec) {
+    case LBM_FP64: return launch_level_step_2d<double>(p, q, fin, fout, h->stream);
+    case LBM_FP32: return launch_level_step_2d<float>(p, q, fin, fout, h->stream);
+    case LBM_FP16_SHIFTED: return launch_level_step_2d<__half>(p, q, fin, fout, h->stream);
+    case LBM_BF16_SHIFTED: return launch_level_step_2d<__nv_bfloat16>(p, q, fin, fout, h->stream);
     }
     return cudaErrorInvalidValue;
 }
@@ -1331,11 +1337,12 @@ static cudaError_t advance_level(lbm_ctx *h, std::vector<StepParams> &params, in
 // from the child at t + 1/2.
 static cudaError_t advance_child(lbm_ctx *h, std::vector<StepParams> &params, int k, int64_t step)
 {
+    const bool three = h->d == 3;  // (in 2D the coupling is part of the child's substeps)
     cudaError_t e = advance_level(h, params, k + 1, 2 * step);
-    if (e == cudaSuccess) e = refine_stage(h, k + 1, 1, 1);
+    if (e == cudaSuccess && three) e = refine_stage(h, k + 1, 1, 1);
     if (e == cudaSuccess) e = advance_level(h, params, k + 1, 2 * step + 1);
-    if (e == cudaSuccess) e = refine_stage(h, k + 1, 1, 0);
-    if (e == cudaSuccess) e = refine_stage(h, k + 1, 2);
+    if (e == cudaSuccess && three) e = refine_stage(h, k + 1, 1, 0);
+    if (e == cudaSuccess && three) e = refine_stage(h, k + 1, 2);
     FineLevel *F = fine_level(h, k + 1);
     F->mcur = 1 - F->mcur;
     return e;
@@ -1355,7 +1362,7 @@ static cudaError_t advance_level(lbm_ctx *h, std::vector<StepParams> &params, in
 {
     const bool child = k < (int)h->levels.size();
     cudaError_t e = cudaSuccess;
-    if (child) e = refine_stage(h, k + 1, 0);
+    if (child && h->d == 3) e = refine_stage(h, k + 1, 0);
     GridRef g = level_grid(h, k);
     params[k].step = step;
     const bool aa = k == 0 && h->pattern == LBM_STREAM_AA;  // (never with refined levels)
@@ -1377,7 +1384,10 @@ static cudaError_t advance_level(lbm_ctx *h, std::vector<StepParams> &params, in
         if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, h->join_ev, 0);
         return e;
     }
-    if (e == cudaSuccess) e = aa ? aa_step(h, params[k]) : launch_update(h, params[k], g.f[*g.cur], g.f[1 - *g.cur]);
+    if (e == cudaSuccess)
+        e = aa ? aa_step(h, params[k])
+               : (k > 0 && h->d == 2 ? launch_level_2d(h, params[k], k, (int)(step & 1))
+                                     : launch_update(h, params[k], g.f[*g.cur], g.f[1 - *g.cur]));
     if (e != cudaSuccess) return e;
     if (!aa) *g.cur = 1 - *g.cur;
     if (!child) return cudaSuccess;

@@ -17,16 +17,19 @@
 // 2 tau_c / tau_f fine -> coarse (leading-order Chapman-Enskog f^neq ~ tau
 // dt grad u with dt_f = dt_c / 2).
 //
-//   k_line_moments : coarse moments on the four interface lines, extended by
-//                    one node past each end (cubic stencils near corners)
-//   k_fill_ring    : fine ring from line moments mixed in time ((1-a) M0 + a M1,
-//                    a = 1/2 at the fine half step) and interpolated in space
-//                    (copy at coincident nodes, (-1, 9, 9, -1)/16 at mid nodes)
-//   k_restrict     : covered coarse ring from the coincident fine node's rho, u
-//                    and its 3 x 3 full-weighted Pi^neq
+//   k_line_moments  : coarse moments at t = 0 on the four interface lines, extended
+//                     by one node past each end (cubic stencils near corners)
+//   k_level_step_2d : a substep of the fine level with its coupling: line moments
+//                     at t + 1; fine ring from line moments mixed in time
+//                     ((1-a) M0 + a M1, a = 1/2 at the fine half step) and
+//                     interpolated in space (copy at coincident nodes,
+//                     (-1, 9, 9, -1)/16 at mid nodes); covered coarse ring from
+//                     the coincident fine node's rho, u and its 3 x 3
+//                     full-weighted Pi^neq
 #pragma once
 
 #include "rr.cuh"
+#include "step.cuh"
 
 namespace rr {
 
@@ -132,108 +135,192 @@ __device__ void store_rebuilt_2d(S *__restrict__ f, int64_t N, int64_t cell, con
     }
 }
 
+// Local moments of the stored coarse field on the interface lines (t = 0)
 template <class S>
-__global__ void k_line_moments(RefineGeom g, const S *__restrict__ fc, const uint8_t *__restrict__ mask,
-                               int streamed, CT<S> *__restrict__ M)
+__global__ void k_line_moments(RefineGeom g, const S *__restrict__ fc, CT<S> *__restrict__ M)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= line_count(g)) return;
     int x, y;
     line_coord(g, e, x, y);
     CT<S> m[6];
-    if (streamed)
-        streamed_moments_2d<S>(fc, mask, g.nxc, g.nyc, x, y, m);
-    else
-        local_moments_2d<S>(fc, g.nxc, g.nyc, x, y, m);
+    local_moments_2d<S>(fc, g.nxc, g.nyc, x, y, m);
 #pragma unroll
     for (int k = 0; k < 6; ++k) M[6 * e + k] = m[k];
 }
 
-template <class C>
-__device__ inline void mix6(const C *__restrict__ M0, const C *__restrict__ M1, C a, int e, C out[6])
-{
-#pragma unroll
-    for (int k = 0; k < 6; ++k) out[k] = (C(1) - a) * M0[6 * e + k] + a * M1[6 * e + k];
-}
+// One substep of a refined 2D level in one launch: the level's own update and,
+// beside it, the coupling with its parent that the substep needs.  Blocks take
+// one of four roles by index (the coupling roles first: their chains of loads
+// are the longest of the launch):
+//   line     (first substep) the parent-side interface moments at t + 1, kept
+//            as the next step's moments at t
+//   ring     the level's ring in the field written, at t + a (a = 1/2, then 1):
+//            line moments mixed in time and interpolated in space.  The first
+//            substep pulls the moments at t + 1 from the parent's pre-step
+//            field itself (the line role stores them in the same launch); the
+//            second reads the stored ones.  Four lanes per ring node, one per
+//            stencil point.
+//   restrict (second substep) the parent's covered ring from the level's
+//            field at t + 1/2, the field this substep's update reads: 16 lanes
+//            per node, one per point of the 3 x 3 filter
+//   update   one thread per cell of the level (update_cell), ring cells fixed
+// None of the roles reads what another writes: ring and restrict write cells
+// that the updates of the two levels leave alone.
+// The coupling is latency-bound (a few thousand nodes).  As launches of its
+// own (line 2.2, ring 2 x 2.9, restrict 15.3 us with one thread per node and
+// its 81 loads in a chain, between two updates of 4.4 us), a coarse step of the
+// 800 x 400 + 641 x 321 cylinder took 35 us; with these two launches of 4.7 us
+// beside the level-0 update it takes 13 us (GB300, FP32).
+struct LevelStep2D {
+    RefineGeom g;
+    int nline, nring, nrestrict;  // blocks of each role
+    const void *parent_old;       // parent field at t (pre-step)
+    void *parent_new;             // parent field at t + 1 (covered ring written)
+    const uint8_t *parent_links, *level_links;  // masks with solids, or null
+    const void *M0;
+    void *M1;
+    double a;                     // time of the ring in the parent step
+    int first;                    // first substep: moments at t + 1 are pulled, and stored by the line role
+    double alpha_down, omega_down, alpha_up, omega_up;
+};
 
-template <class S>
-__global__ void k_fill_ring(RefineGeom g, const CT<S> *__restrict__ M0, const CT<S> *__restrict__ M1, CT<S> a,
-                            CT<S> alpha, CT<S> omega, S *__restrict__ ff)
+// Ring node t of an nfx x nfy level
+__device__ inline void ring_coord(int nfx, int nfy, int t, int &i, int &j)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int nfx = g.nfx, nfy = g.nfy;
-    const int count = 2 * nfx + 2 * (nfy - 2);
-    if (t >= count) return;
-    int i, j;
     if (t < nfx) { i = t; j = 0; }
     else if (t < 2 * nfx) { i = t - nfx; j = nfy - 1; }
     else if (t < 2 * nfx + nfy - 2) { i = 0; j = 1 + t - 2 * nfx; }
     else { i = nfx - 1; j = 1 + t - 2 * nfx - (nfy - 2); }
+}
+__host__ __device__ inline int ring_count(int nfx, int nfy) { return 2 * nfx + 2 * (nfy - 2); }
+
+constexpr int kLevelBlock = 128;
+
+template <class S>
+__device__ __forceinline__ void level_line(const LevelStep2D &q, int e)
+{
     using C = CT<S>;
-    const bool on_h = (j == 0 || j == nfy - 1);
-    const C am = a;
+    if (e >= line_count(q.g)) return;
+    int x, y;
+    line_coord(q.g, e, x, y);
     C m[6];
-    if (on_h) {
-        const int top = j == 0 ? 0 : 1;
-        if ((i & 1) == 0) {
-            mix6<C>(M0, M1, am, entry_h(g, g.X0 + i / 2, top), m);
-        } else {
-            const int xa = g.X0 + (i - 1) / 2;
-            C t0[6], t1[6], t2[6], t3[6];
-            mix6<C>(M0, M1, am, entry_h(g, xa - 1, top), t0);
-            mix6<C>(M0, M1, am, entry_h(g, xa, top), t1);
-            mix6<C>(M0, M1, am, entry_h(g, xa + 1, top), t2);
-            mix6<C>(M0, M1, am, entry_h(g, xa + 2, top), t3);
+    streamed_moments_2d<S>((const S *)q.parent_old, q.parent_links, q.g.nxc, q.g.nyc, x, y, m);
 #pragma unroll
-            for (int k = 0; k < 6; ++k) m[k] = (-t0[k] + C(9) * t1[k] + C(9) * t2[k] - t3[k]) * C(0.0625);
-        }
-    } else {
-        const int right = i == 0 ? 0 : 1;
-        if ((j & 1) == 0) {
-            mix6<C>(M0, M1, am, entry_v(g, g.Y0 + j / 2, right), m);
-        } else {
-            const int ya = g.Y0 + (j - 1) / 2;
-            C t0[6], t1[6], t2[6], t3[6];
-            mix6<C>(M0, M1, am, entry_v(g, ya - 1, right), t0);
-            mix6<C>(M0, M1, am, entry_v(g, ya, right), t1);
-            mix6<C>(M0, M1, am, entry_v(g, ya + 1, right), t2);
-            mix6<C>(M0, M1, am, entry_v(g, ya + 2, right), t3);
-#pragma unroll
-            for (int k = 0; k < 6; ++k) m[k] = (-t0[k] + C(9) * t1[k] + C(9) * t2[k] - t3[k]) * C(0.0625);
-        }
-    }
-    store_rebuilt_2d<S>(ff, (int64_t)nfx * nfy, i + (int64_t)nfx * j, m, alpha, omega);
+    for (int k = 0; k < 6; ++k) ((C *)q.M1)[6 * e + k] = m[k];
 }
 
 template <class S>
-__global__ void k_restrict(RefineGeom g, const S *__restrict__ ff_prev, const uint8_t *__restrict__ fmask,
-                           CT<S> alpha, CT<S> omega, S *__restrict__ fc)
+__device__ __forceinline__ void level_ring(const LevelStep2D &q, int lane_id, S *ff)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int w = g.Wc - 1, h = g.Hc - 1;  // ring of the rectangle [X0+1, X0+Wc-1] x [Y0+1, Y0+Hc-1]
-    const int count = 2 * w + 2 * (h - 2);
-    if (t >= count) return;
-    int x, y;
-    if (t < w) { x = g.X0 + 1 + t; y = g.Y0 + 1; }
-    else if (t < 2 * w) { x = g.X0 + 1 + (t - w); y = g.Y0 + g.Hc - 1; }
-    else if (t < 2 * w + h - 2) { x = g.X0 + 1; y = g.Y0 + 2 + (t - 2 * w); }
-    else { x = g.X0 + g.Wc - 1; y = g.Y0 + 2 + (t - 2 * w - (h - 2)); }
     using C = CT<S>;
-    const int i = 2 * (x - g.X0), j = 2 * (y - g.Y0);
-    const C w3[3] = {C(1), C(2), C(1)};
-    C mc[6] = {C(0), C(0), C(0), C(0), C(0), C(0)}, m[6];
+    const RefineGeom &g = q.g;
+    const int t = lane_id >> 2, r = lane_id & 3;
+    const bool node = t < ring_count(g.nfx, g.nfy);  // other lanes still join the shuffles
+    int i = 0, j = 0;
+    if (node) ring_coord(g.nfx, g.nfy, t, i, j);
+    const bool on_h = j == 0 || j == g.nfy - 1;
+    const int c = on_h ? i : j;           // fine coordinate along the line
+    const int side = on_h ? (j != 0) : (i != 0);
+    const bool odd = c & 1;
+    // lane r: stencil point (c - 1)/2 - 1 + r of an odd node; the coincident
+    // parent node (lane 0) of an even one
+    const int k = odd ? (c - 1) / 2 - 1 + r : c / 2;
+    C m[6];
 #pragma unroll
-    for (int l = -1; l <= 1; ++l)
+    for (int s = 0; s < 6; ++s) m[s] = C(0);
+    if (node && (odd || r == 0)) {
+        const int e = on_h ? entry_h(g, g.X0 + k, side) : entry_v(g, g.Y0 + k, side);
+        C m1[6];
+        if (q.first) {
+            const int x = on_h ? g.X0 + k : g.X0 + side * g.Wc, y = on_h ? g.Y0 + side * g.Hc : g.Y0 + k;
+            streamed_moments_2d<S>((const S *)q.parent_old, q.parent_links, g.nxc, g.nyc, x, y, m1);
+        } else {
 #pragma unroll
-        for (int k = -1; k <= 1; ++k) {
-            streamed_moments_2d<S>(ff_prev, fmask, g.nfx, g.nfy, i + k, j + l, m);
-            const C wt = w3[k + 1] * w3[l + 1] * C(0.0625);
-            mc[3] += wt * m[3];
-            mc[4] += wt * m[4];
-            mc[5] += wt * m[5];
-            if (k == 0 && l == 0) { mc[0] = m[0]; mc[1] = m[1]; mc[2] = m[2]; }
+            for (int s = 0; s < 6; ++s) m1[s] = ((const C *)q.M1)[6 * e + s];
         }
-    store_rebuilt_2d<S>(fc, (int64_t)g.nxc * g.nyc, x + (int64_t)g.nxc * y, mc, alpha, omega);
+        const C a = C(q.a);
+#pragma unroll
+        for (int s = 0; s < 6; ++s) m[s] = (C(1) - a) * ((const C *)q.M0)[6 * e + s] + a * m1[s];
+    }
+    C v[6];
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        const C t1 = __shfl_down_sync(0xffffffffu, m[s], 1), t2 = __shfl_down_sync(0xffffffffu, m[s], 2),
+                t3 = __shfl_down_sync(0xffffffffu, m[s], 3);
+        v[s] = odd ? (-m[s] + C(9) * t1 + C(9) * t2 - t3) * C(0.0625) : m[s];
+    }
+    if (node && r == 0)
+        store_rebuilt_2d<S>(ff, (int64_t)g.nfx * g.nfy, i + (int64_t)g.nfx * j, v, C(q.alpha_down), C(q.omega_down));
+}
+
+template <class S>
+__device__ __forceinline__ void level_restrict(const LevelStep2D &q, int lane_id, const S *ff_prev)
+{
+    using C = CT<S>;
+    const RefineGeom &g = q.g;
+    const int w = g.Wc - 1, h = g.Hc - 1;  // ring of the rectangle [X0+1, X0+Wc-1] x [Y0+1, Y0+Hc-1]
+    const int t = lane_id >> 4, l = lane_id & 15;
+    const bool node = t < ring_count(w, h);  // other lanes still join the shuffles
+    int a = 0, b = 0;
+    if (node) ring_coord(w, h, t, a, b);
+    const int x = g.X0 + 1 + a, y = g.Y0 + 1 + b;
+    C m[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) m[k] = C(0);
+    if (node && l < 9)
+        streamed_moments_2d<S>(ff_prev, q.level_links, g.nfx, g.nfy, 2 * (x - g.X0) + l % 3 - 1,
+                               2 * (y - g.Y0) + l / 3 - 1, m);
+    C mc[6] = {C(0), C(0), C(0), C(0), C(0), C(0)};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) mc[k] = __shfl_sync(0xffffffffu, m[k], 4, 16);
+#pragma unroll
+    for (int s = 0; s < 9; ++s) {
+        const C wt = C((s % 3 == 1 ? 2 : 1) * (s / 3 == 1 ? 2 : 1)) * C(0.0625);
+#pragma unroll
+        for (int k = 3; k < 6; ++k) mc[k] += wt * __shfl_sync(0xffffffffu, m[k], s, 16);
+    }
+    if (node && l == 0)
+        store_rebuilt_2d<S>((S *)q.parent_new, (int64_t)g.nxc * g.nyc, x + (int64_t)g.nxc * y, mc, C(q.alpha_up),
+                            C(q.omega_up));
+}
+
+template <class S, int MASK>
+__global__ void __launch_bounds__(kLevelBlock)
+    k_level_step_2d(const __grid_constant__ StepParams p, const __grid_constant__ LevelStep2D q)
+{
+    using C = CT<S>;
+    int b = blockIdx.x;
+    const int tid = threadIdx.x;
+    if (b < q.nline) return level_line<S>(q, b * kLevelBlock + tid);
+    b -= q.nline;
+    if (b < q.nring) return level_ring<S>(q, b * kLevelBlock + tid, (S *)p.out[0]);
+    b -= q.nring;
+    if (b < q.nrestrict) return level_restrict<S>(q, b * kLevelBlock + tid, (const S *)p.in[0]);
+    b -= q.nrestrict;
+    const unsigned t = (unsigned)b * kLevelBlock + tid;
+    if (t >= (unsigned)p.ncell) return;
+    const unsigned nx = p.n[0], y = t / nx;
+    update_cell<D2Q9, S, C, false, MASK>(p, p.in, p.out, (int)(t - y * nx), (int)y, 0);
+}
+
+// Launch one substep of a refined 2D level (fin read, fout written)
+template <class S>
+cudaError_t launch_level_step_2d(const StepParams &p, const LevelStep2D &q0, const void *fin, void *fout, cudaStream_t st)
+{
+    StepParams s = p;
+    set_bases<D2Q9, S>(s, fin, fout);
+    LevelStep2D q = q0;
+    auto blocks = [](int64_t threads) { return (int)((threads + kLevelBlock - 1) / kLevelBlock); };
+    q.nline = q.first ? blocks(line_count(q.g)) : 0;
+    q.nring = blocks(4 * (int64_t)ring_count(q.g.nfx, q.g.nfy));
+    q.nrestrict = q.first ? 0 : blocks(16 * (int64_t)ring_count(q.g.Wc - 1, q.g.Hc - 1));
+    const unsigned grid = (unsigned)(q.nline + q.nring + q.nrestrict + blocks(p.ncell));
+    if (p.any_solid)
+        k_level_step_2d<S, kMaskLinks><<<grid, kLevelBlock, 0, st>>>(s, q);
+    else
+        k_level_step_2d<S, kMaskSkip><<<grid, kLevelBlock, 0, st>>>(s, q);
+    return cudaGetLastError();
 }
 
 // ===========================================================================

@@ -46,3 +46,37 @@ def test_default_block_leaves_no_idle_warp_and_changes_nothing(lattice, nx, bloc
     ref, _ = populations(c, "fp16", (64, 2))
     assert got == (block, 2)
     assert np.array_equal(f, ref)
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("fp32", 1e-5)])
+@pytest.mark.parametrize("ext", [(4, 4), (5, 4), (4, 33), (67, 5)])
+def test_level_step_2d_on_small_and_long_patches(ext, prec, tol):
+    """The refined level's substep with its coupling at the smallest ring, odd
+    extents and long sides (rings that end inside a block of every role),
+    against the oracle; both levels after three coarse steps."""
+    import oracle
+    from cases import to_oracle
+    from paper_1710_02065_gb300 import inputs, lbm
+    n, patch = (80, 44, 1), (3, 4, *ext)
+    nf = (2 * ext[0] + 1, 2 * ext[1] + 1)
+    c = Case("patch", D2Q9, n, 0.6)
+    c.rho0, c.u0 = inputs.uniform_flow_perturbed(n[0], n[1], 0.05, 4, rel=0.2)
+    rho_f, u_f = inputs.uniform_flow_perturbed(*nf, 0.05, 5, rel=0.2)
+    P, _ = to_oracle(c)
+    T = oracle.TwoLevel(P, *patch)
+    T.init(c.rho0, c.u0, rho_f, u_f)
+    s = to_gpu(c, PRECS[prec])
+    lbm.lbm_add_refinement_patch(s.h, (*patch[:2], 0), (*ext, 1))
+    lbm.lbm_set_state_level(s.h, 1, rho_f, u_f)
+    lbm.lbm_set_state(s.h, c.rho0, c.u0)
+    T.run(3)
+    s.step(3)
+    live = np.ones((n[1], n[0]), bool)
+    live[patch[1] + 2:patch[1] + ext[1] - 1, patch[0] + 2:patch[0] + ext[0] - 1] = False  # frozen covered cells
+    for level, (Q, f, keep) in enumerate(((T.Pc, T.fc, live.reshape(-1)), (T.Pf, T.ff, slice(None)))):
+        r, u, _ = Q.moments(f)
+        gr, gu = np.zeros(Q.ncell), np.zeros((Q.ncell, 3))
+        lbm.lbm_moments_level(s.h, level, gr, gu, None)
+        assert np.linalg.norm((gr - r)[keep]) <= tol * np.linalg.norm(r[keep])
+        assert np.linalg.norm((gu - u)[keep]) <= tol * np.linalg.norm(u[keep])
+    s.close()
