@@ -28,6 +28,8 @@ struct FineLevel {
     int cur = 0;
     uint8_t *mask_d = nullptr;           // ring fixed + user solids
     bool has_solid = false;              // the mask holds solid cells
+    int *near_d = nullptr;               // fluid cells next to a solid (the force's links start there)
+    int nnear = 0;
     std::vector<uint8_t> user_mask;      // user solids (host copy)
     RefineGeom geom{};                   // position in the parent level's nodes
     double *M[2] = {nullptr, nullptr};   // parent-side interface moments at t and t + 1 (compute type; sized for FP64)
@@ -51,6 +53,8 @@ struct lbm_ctx {
     int cur = 0;
     uint8_t *solid_d = nullptr;
     bool has_solid = false;  // level 0's mask holds solid cells (else only fixed ones)
+    int *near_d = nullptr;   // level 0's fluid cells next to a solid
+    int nnear = 0;
     double *prof_d[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     int kind[6] = {0, 0, 0, 0, 0, 0};
     double u_face[6][3] = {};
@@ -70,6 +74,7 @@ struct lbm_ctx {
     int staging = -1;     // row-staged kernel: -1 default (off), 0 off, 1 on where eligible
     int stages = 0;       // its shared-memory stages (0: 2)
     int rows_block = 0;   // its threads per CTA (0: automatic)
+    unsigned *done_d = nullptr;  // block counter of the force sum (zero between launches)
     unsigned *err_d = nullptr;  // device error word of the row-staged kernel (bounded waits)
     uint64_t rows_wait_ns = 2000000000ull;  // limit of each of its waits for a tile's copies
     int collision = LBM_COLLISION_RR;
@@ -126,6 +131,8 @@ struct GridRef {
     void **f;
     int *cur;
     const uint8_t *mask;
+    const int *near;  // fluid cells next to a solid
+    int nnear;
 };
 
 static const double *shift_of(const lbm_ctx *h, const GridRef &g)
@@ -135,7 +142,7 @@ static const double *shift_of(const lbm_ctx *h, const GridRef &g)
 
 static GridRef coarse_ref(lbm_ctx *h)
 {
-    return GridRef{{h->n[0], h->n[1], h->n[2]}, h->ncell, h->f, &h->cur, h->solid_d};
+    return GridRef{{h->n[0], h->n[1], h->n[2]}, h->ncell, h->f, &h->cur, h->solid_d, h->near_d, h->nnear};
 }
 static int nlevels(const lbm_ctx *h) { return 1 + (int)h->levels.size(); }
 static FineLevel *fine_level(lbm_ctx *h, int k) { return h->levels[(size_t)k - 1]; }  // k >= 1
@@ -143,7 +150,7 @@ static GridRef level_grid(lbm_ctx *h, int k)
 {
     if (k == 0) return coarse_ref(h);
     FineLevel *F = fine_level(h, k);
-    return GridRef{{F->n[0], F->n[1], F->n[2]}, F->ncell, F->f, &F->cur, F->mask_d};
+    return GridRef{{F->n[0], F->n[1], F->n[2]}, F->ncell, F->f, &F->cur, F->mask_d, F->near_d, F->nnear};
 }
 static double level_tau(lbm_ctx *h, int k) { return k == 0 ? h->tau : fine_level(h, k)->tau; }
 // Bytes of one interface-moment buffer of a refined level (sized for FP64)
@@ -283,14 +290,13 @@ struct Reduce {
 };
 template <class L, class S>
 struct Force {
+    // F (device, 3 doubles); partial: 3 doubles per block; done: block counter, zero between launches
     static cudaError_t run(cudaStream_t st, const int *n, const int *per, const void *f, const uint8_t *mask,
-                           double *partial, int nblocks, const double *dsh)
+                           const int *cells, int count, int blocks, double *partial, unsigned *done, double *F,
+                           const double *dsh)
     {
-        k_force<L, S><<<nblocks, RED_BLOCK, 0, st>>>(n[0], n[1], n[2], per[0], per[1], per[2], (const S *)f, mask,
-                                                      partial, dsh);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_reduce_final<<<1, 32 * RED_FIELDS, 0, st>>>(nblocks, partial, partial + (int64_t)nblocks * RED_FIELDS);
+        k_force<L, S><<<blocks, kForceBlock, 0, st>>>(n[0], n[1], n[2], per[0], per[1], per[2], (const S *)f, mask,
+                                                      cells, count, partial, done, F, dsh);
         return cudaGetLastError();
     }
 };
@@ -440,6 +446,8 @@ static void release(lbm_ctx *h)
         if (h->prof_d[k]) cudaFree(h->prof_d[k]);
     if (h->red_d) cudaFree(h->red_d);
     if (h->err_d) cudaFree(h->err_d);
+    if (h->done_d) cudaFree(h->done_d);
+    if (h->near_d) cudaFree(h->near_d);
     if (h->chi_tab_f) cudaFree(h->chi_tab_f);
     if (h->stage_d) cudaFree(h->stage_d);
     if (h->bad_d) cudaFree(h->bad_d);
@@ -458,6 +466,7 @@ static void release(lbm_ctx *h)
             if (F->M[k]) cudaFree(F->M[k]);
         }
         if (F->mask_d) cudaFree(F->mask_d);
+        if (F->near_d) cudaFree(F->near_d);
         delete F;
     }
     delete h;
@@ -520,6 +529,12 @@ extern "C" int lbm_create(lbm_handle *out, int lattice, const int extents[3], do
         cudaGetLastError();
         release(h);
         return fail(nullptr, LBM_ENOMEM, "cudaMalloc of the error word failed");
+    }
+    if (cudaMalloc(&h->done_d, sizeof(unsigned)) != cudaSuccess ||
+        cudaMemsetAsync(h->done_d, 0, sizeof(unsigned), h->stream) != cudaSuccess) {
+        cudaGetLastError();
+        release(h);
+        return fail(nullptr, LBM_ENOMEM, "cudaMalloc of the force counter failed");
     }
     if (upload_sponge_tables(h) != LBM_OK) {
         cudaGetLastError();
@@ -597,7 +612,10 @@ static int upload_level_mask(lbm_ctx *h, int k)
     const std::vector<uint8_t> &user = k == 0 ? h->user_mask : fine_level(h, k)->user_mask;
     if (k == 0 && user.empty() && !has_child) {
         if (h->solid_d) cudaFree(h->solid_d);
+        if (h->near_d) cudaFree(h->near_d);
         h->solid_d = nullptr;
+        h->near_d = nullptr;
+        h->nnear = 0;
         h->has_solid = false;
         return LBM_OK;
     }
@@ -626,7 +644,22 @@ static int upload_level_mask(lbm_ctx *h, int k)
     uint8_t *&dst = k == 0 ? h->solid_d : fine_level(h, k)->mask_d;
     if (!dst) CUDA_TRY(h, cudaMalloc(&dst, (size_t)g.ncell));
     CUDA_TRY(h, cudaMemcpyAsync(dst, m.data(), (size_t)g.ncell, cudaMemcpyHostToDevice, h->stream));
+    // the fluid cells next to a solid, for the force
+    std::vector<int> near;
+    for (size_t c = 0; c < m.size(); ++c)
+        if ((m[c] & MASK_TYPE) == 0 && (m[c] & MASK_NEAR_SOLID)) near.push_back((int)c);
+    int *&nd = k == 0 ? h->near_d : fine_level(h, k)->near_d;
+    int &nn = k == 0 ? h->nnear : fine_level(h, k)->nnear;
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+    if (nd) CUDA_TRY(h, cudaFree(nd));
+    nd = nullptr;
+    nn = 0;
+    if (!near.empty()) {
+        CUDA_TRY(h, cudaMalloc(&nd, sizeof(int) * near.size()));
+        CUDA_TRY(h, cudaMemcpyAsync(nd, near.data(), sizeof(int) * near.size(), cudaMemcpyHostToDevice, h->stream));
+        CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+        nn = (int)near.size();
+    }
     return LBM_OK;
 }
 
@@ -1578,6 +1611,29 @@ static int level_ref(lbm_ctx *h, int level, GridRef &g)
     return LBM_OK;
 }
 
+// Enqueue the force on level `level` into F_dev (device, 3 doubles)
+static int enqueue_force(lbm_ctx *h, int level, double *F_dev)
+{
+    GridRef g;
+    int rc = level_ref(h, level, g);
+    if (rc != LBM_OK) return rc;
+    cudaError_t e;
+    if (!g.mask || g.nnear == 0) {
+        e = cudaMemsetAsync(F_dev, 0, 3 * sizeof(double), h->stream);
+    } else {
+        int per[3] = {1, 1, 1};
+        if (level == 0)
+            for (int a = 0; a < 3; ++a) per[a] = h->kind[2 * a] == LBM_BC_PERIODIC ? 1 : 0;
+        const int blocks = std::min((g.nnear + kForceBlock - 1) / kForceBlock, h->red_blocks);
+        e = dispatch<Force>(h->lattice, h->prec, h->stream, (const int *)g.n, (const int *)per,
+                            (const void *)g.f[*g.cur], g.mask, g.near, g.nnear, blocks, h->red_d, h->done_d, F_dev,
+                            shift_of(h, g));
+        h->launches += 1;
+    }
+    if (e != cudaSuccess) return fail(h, LBM_ECUDA, "force: %s", cudaGetErrorString(e));
+    return LBM_OK;
+}
+
 extern "C" int lbm_force(lbm_handle h, int level, double F[3])
 {
     CHECK_HANDLE(h);
@@ -1586,22 +1642,12 @@ extern "C" int lbm_force(lbm_handle h, int level, double F[3])
         if (rc0 != LBM_OK) return rc0;
     }
     if (!F) return fail(h, LBM_EINVAL, "F is null");
-    GridRef g;
-    int rc = level_ref(h, level, g);
+    double *F_dev = h->red_d + (size_t)h->red_blocks * RED_FIELDS;
+    const int rc = enqueue_force(h, level, F_dev);
     if (rc != LBM_OK) return rc;
-    F[0] = F[1] = F[2] = 0.0;
-    if (!g.mask) return LBM_OK;
-    int per[3] = {1, 1, 1};
-    if (level == 0)
-        for (int a = 0; a < 3; ++a) per[a] = h->kind[2 * a] == LBM_BC_PERIODIC ? 1 : 0;
-    double out[RED_FIELDS];
-    cudaError_t e = dispatch<Force>(h->lattice, h->prec, h->stream, (const int *)g.n, (const int *)per,
-                                    (const void *)g.f[*g.cur], g.mask, h->red_d, h->red_blocks, shift_of(h, g));
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, h->red_d + (size_t)h->red_blocks * RED_FIELDS, sizeof out, cudaMemcpyDeviceToHost,
-                            h->stream);
+    double out[3];
+    cudaError_t e = cudaMemcpyAsync(out, F_dev, sizeof out, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    h->launches += 2;
     if (e != cudaSuccess) return fail(h, LBM_ECUDA, "lbm_force: %s", cudaGetErrorString(e));
     for (int a = 0; a < 3; ++a) F[a] = out[a];
     return LBM_OK;
@@ -1615,25 +1661,7 @@ extern "C" int lbm_force_async(lbm_handle h, int level, double *F_dev)
         if (rc0 != LBM_OK) return rc0;
     }
     if (!F_dev) return fail(h, LBM_EINVAL, "F_dev is null");
-    GridRef g;
-    int rc = level_ref(h, level, g);
-    if (rc != LBM_OK) return rc;
-    cudaError_t e;
-    if (!g.mask) {
-        e = cudaMemsetAsync(F_dev, 0, 3 * sizeof(double), h->stream);
-    } else {
-        int per[3] = {1, 1, 1};
-        if (level == 0)
-            for (int a = 0; a < 3; ++a) per[a] = h->kind[2 * a] == LBM_BC_PERIODIC ? 1 : 0;
-        e = dispatch<Force>(h->lattice, h->prec, h->stream, (const int *)g.n, (const int *)per,
-                            (const void *)g.f[*g.cur], g.mask, h->red_d, h->red_blocks, shift_of(h, g));
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(F_dev, h->red_d + (size_t)h->red_blocks * RED_FIELDS, 3 * sizeof(double),
-                                cudaMemcpyDeviceToDevice, h->stream);
-        h->launches += 2;
-    }
-    if (e != cudaSuccess) return fail(h, LBM_ECUDA, "lbm_force_async: %s", cudaGetErrorString(e));
-    return LBM_OK;
+    return enqueue_force(h, level, F_dev);
 }
 
 extern "C" int lbm_level_info(lbm_handle h, int level, int extents[3], double *tau)

@@ -80,3 +80,40 @@ def test_level_step_2d_on_small_and_long_patches(ext, prec, tol):
         assert np.linalg.norm((gr - r)[keep]) <= tol * np.linalg.norm(r[keep])
         assert np.linalg.norm((gu - u)[keep]) <= tol * np.linalg.norm(u[keep])
     s.close()
+
+
+@pytest.mark.parametrize("lattice,n,solids", [(D2Q9, (9, 9, 1), "cell"), (D2Q9, (40, 9, 1), "wall"),
+                                              (D3Q19, (9, 8, 7), "cell"), (D3Q27, (160, 130, 5), "wall")])
+def test_force_sums_every_link(lattice, n, solids):
+    """Lists of fewer cells than a block, not a whole number of blocks, and
+    more than one turn of the largest grid (41,600 cells next to a wall);
+    twice in a row, so that the block counter is seen to be back at zero.  The
+    sums have at most 1.9 M terms of magnitude < 0.6: 1e-10 absolute covers
+    their FP64 round-off.  The reference is the exact sum over the links (the
+    oracle adds them one after the other, which alone loses 1e-10 here)."""
+    import math
+    import oracle
+    from cases import to_oracle
+    from paper_1710_02065_gb300 import lbm
+    c = with_random_state(Case("force", lattice, n, 0.6), seed=6, spread=0.3)
+    m = np.zeros((n[2], n[1], n[0]), np.uint8)
+    if solids == "cell":
+        m[n[2] // 2, 4, 4] = 1
+    else:
+        m[n[2] // 2, n[1] // 2 if lattice == D2Q9 else slice(None), :] = 1
+    c.solid = m.reshape(-1)
+    P, f = to_oracle(c)
+    _, q, xi, _, _ = oracle.lattice(lattice)
+    sums = [math.fsum(f[i].reshape(m.shape)[(np.roll(m, -xi[i][::-1], (0, 1, 2)) == 1) & (m == 0)]) for i in range(q)]
+    ref = np.array([math.fsum(2.0 * xi[i][a] * sums[i] for i in range(q)) for a in range(3)])
+    assert np.abs(P.wall_force(f) - ref).max() < 1e-8
+    s = to_gpu(c, PRECS["fp64"])
+    for _ in range(2):
+        assert np.abs(lbm.lbm_force(s.h, 0) - ref).max() < 1e-10
+    dev = torch.full((3,), 7.0, dtype=torch.float64, device="cuda")
+    lbm.lbm_force_async(s.h, 0, dev.data_ptr())
+    lbm.lbm_sync(s.h)
+    assert np.abs(dev.cpu().numpy() - ref).max() < 1e-10
+    lbm.lbm_set_geometry(s.h, None)
+    assert not lbm.lbm_force(s.h, 0).any()
+    s.close()
