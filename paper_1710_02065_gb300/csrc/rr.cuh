@@ -181,6 +181,24 @@ struct Store<__nv_bfloat16> {
 __device__ __forceinline__ float fmac(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fmac(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// A product rounded on its own, never fused into a sum that uses it.  Left to
+// the compiler, which products of a sum are fused depended on the code around
+// an inlined copy, so the same cell could round differently in two kernels
+// (16-bit storage and p' show such differences); in the collision every
+// product that a plain sum uses is written with mulr, every fused one with
+// fmac.  D3Q27, whose generic pair rebuild is left to the compiler, keeps the
+// plain product.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <class L, class C>
+__device__ __forceinline__ C mulr(C a, C b)
+{
+    if constexpr (full_third_order<L>())
+        return a * b;
+    else
+        return mul_rn(a, b);
+}
+
 // Device cell-type byte: bits 0-1 the cell type (0 fluid, 1 solid wall,
 // 2 fixed), bit 2 set when a lattice neighbour is a solid wall.
 constexpr uint8_t MASK_TYPE = 3, MASK_SOLID = 1, MASK_NEAR_SOLID = 4;
@@ -599,74 +617,59 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 //                                         T_y = A_xxy + A_yzz, T_z = A_xxz + A_yyz),
 //   edge s_a e_a + s_b e_b:  9 w2 (s_b A_aab + s_a A_abb),
 // which is what the pair sums and differences of rebuild_pair evaluate to.
-// O4 = false drops the optional fourth-order D2Q9 term.  D3Q27 uses the
-// generic pair rebuild.
+// O4 = false drops the optional fourth-order D2Q9 term.  VEC: which product of
+// a1_a / 12 +- a1_b / 12 is fused: one choice in the single-lattice vector
+// kernels, the other in the general and the batched ones.  D3Q27 uses the generic pair rebuild.
 // ---------------------------------------------------------------------------
-template <class L, class C, bool O4 = true>
+template <class L, class C, bool O4 = true, bool VEC = false>
 __device__ __forceinline__ void rebuild_all(const Coef<C> &k, C *o)
 {
     if constexpr (L::Q == 19) {
         // w0 = 1/3, w1 = 1/18, w2 = 1/36; 4.5 w1 = 1/4, 4.5 w2 = 1/8, 9 w2 = 1/4
         const C tr = (k.xx + k.yy) + k.zz;
-        const C tr3 = tr * C(1.0 / 3.0), t23 = tr - tr3;
+        const C tr3 = mulr<L>(tr, C(1.0 / 3.0)), t23 = tr - tr3;
         o[0] = fmac(C(-1.5), tr3, C(1.0 / 3.0) * k.a0);
         const C wa1 = C(1.0 / 18.0) * k.a0, wa2 = C(1.0 / 36.0) * k.a0;
         // faces: E = w1 a0 + (A_aa - tr/3) / 4, O = a1_a / 6 - T_a / 2
-        {
-            const C E = fmac(C(0.25), k.xx - tr3, wa1);
-            const C O = fmac(C(-0.5), k.xzz + k.xyy, C(1.0 / 6.0) * k.a1x);
-            o[1] = E + O;
-            o[10] = E - O;
-        }
-        {
-            const C E = fmac(C(0.25), k.yy - tr3, wa1);
-            const C O = fmac(C(-0.5), k.xxy + k.yzz, C(1.0 / 6.0) * k.a1y);
-            o[2] = E + O;
-            o[11] = E - O;
-        }
-        {
-            const C E = fmac(C(0.25), k.zz - tr3, wa1);
-            const C O = fmac(C(-0.5), k.yyz + k.xxz, C(1.0 / 6.0) * k.a1z);
-            o[3] = E + O;
-            o[12] = E - O;
-        }
-        // edges: a1 / 12 shared by the three planes
-        const C jx = C(1.0 / 12.0) * k.a1x, jy = C(1.0 / 12.0) * k.a1y, jz = C(1.0 / 12.0) * k.a1z;
-        {  // xy plane: 4 (1,1,0) / 13, 5 (1,-1,0) / 14
-            const C base = fmac(C(0.125), t23 - k.zz, wa2);
-            const C Ep = fmac(C(0.25), k.xy, base), Em = fmac(C(-0.25), k.xy, base);
-            const C Op = fmac(C(0.25), k.xxy + k.xyy, jx + jy);
-            const C Om = fmac(C(0.25), k.xyy - k.xxy, jx - jy);
-            o[4] = Ep + Op;
-            o[13] = Ep - Op;
-            o[5] = Em + Om;
-            o[14] = Em - Om;
-        }
-        {  // xz plane: 6 (1,0,1) / 15, 7 (1,0,-1) / 16
-            const C base = fmac(C(0.125), t23 - k.yy, wa2);
-            const C Ep = fmac(C(0.25), k.xz, base), Em = fmac(C(-0.25), k.xz, base);
-            const C Op = fmac(C(0.25), k.xzz + k.xxz, jx + jz);
-            const C Om = fmac(C(0.25), k.xzz - k.xxz, jx - jz);
-            o[6] = Ep + Op;
-            o[15] = Ep - Op;
-            o[7] = Em + Om;
-            o[16] = Em - Om;
-        }
-        {  // yz plane: 8 (0,1,1) / 17, 9 (0,1,-1) / 18
-            const C base = fmac(C(0.125), t23 - k.xx, wa2);
-            const C Ep = fmac(C(0.25), k.yz, base), Em = fmac(C(-0.25), k.yz, base);
-            const C Op = fmac(C(0.25), k.yzz + k.yyz, jy + jz);
-            const C Om = fmac(C(0.25), k.yzz - k.yyz, jy - jz);
-            o[8] = Ep + Op;
-            o[17] = Ep - Op;
-            o[9] = Em + Om;
-            o[18] = Em - Om;
-        }
+        auto face = [&](int i, C Aaa, C a1, C T) {
+            const C E = fmac(C(0.25), Aaa - tr3, wa1);
+            const C O = fmac(C(-0.5), T, C(1.0 / 6.0) * a1);
+            o[i] = E + O;
+            o[i + 9] = E - O;
+        };
+        face(1, k.xx, k.a1x, k.xzz + k.xyy);
+        face(2, k.yy, k.a1y, k.xxy + k.yzz);
+        face(3, k.zz, k.a1z, k.yyz + k.xxz);
+        // edges of the planes (a, b): i (1, 1) / i + 9, i + 1 (1, -1) / i + 10; the odd
+        // part's first order is a1_a / 12 +- a1_b / 12
+        constexpr C w12 = C(1.0 / 12.0);
+        auto plane = [&](int i, C Acc, C Aab, C a1a, C a1b, C Tp, C Tm) {
+            const C base = fmac(C(0.125), t23 - Acc, wa2);
+            const C Ep = fmac(C(0.25), Aab, base), Em = fmac(C(-0.25), Aab, base);
+            C jp, jm;
+            if (VEC) {
+                const C ja = mulr<L>(w12, a1a);
+                jp = fmac(w12, a1b, ja);
+                jm = fmac(-w12, a1b, ja);
+            } else {
+                const C jb = mulr<L>(w12, a1b);
+                jp = i == 8 ? (mulr<L>(w12, a1a) + jb) : fmac(w12, a1a, jb);
+                jm = i == 8 ? (mulr<L>(w12, a1a) - jb) : fmac(w12, a1a, -jb);
+            }
+            const C Op = fmac(C(0.25), Tp, jp), Om = fmac(C(0.25), Tm, jm);
+            o[i] = Ep + Op;
+            o[i + 9] = Ep - Op;
+            o[i + 1] = Em + Om;
+            o[i + 10] = Em - Om;
+        };
+        plane(4, k.zz, k.xy, k.a1x, k.a1y, k.xxy + k.xyy, k.xyy - k.xxy);
+        plane(6, k.yy, k.xz, k.a1x, k.a1z, k.xzz + k.xxz, k.xzz - k.xxz);
+        plane(8, k.xx, k.yz, k.a1y, k.a1z, k.yzz + k.yyz, k.yzz - k.yyz);
     } else if constexpr (L::Q == 9) {
         // w0 = 4/9, w1 = 1/9, w2 = 1/36; H_xxyy / (4 c_s^8) weighted: rest 1,
         // faces -1/2, diagonals 1/4 (zero coefficient unless fourth order)
         const C tr = k.xx + k.yy;
-        const C tr3 = tr * C(1.0 / 3.0);
+        const C tr3 = mulr<L>(tr, C(1.0 / 3.0));
         C g0 = fmac(C(-2.0), tr3, C(4.0 / 9.0) * k.a0);
         if (O4) g0 = g0 + k.xxyy;
         o[0] = g0;
@@ -688,10 +691,20 @@ __device__ __forceinline__ void rebuild_all(const Coef<C> &k, C *o)
         {  // 3 (1,1) / 7, 4 (-1,1) / 8
             C base = fmac(C(0.125), tr - tr3, wa2);
             if (O4) base = fmac(C(0.25), k.xxyy, base);
-            const C jx = C(1.0 / 12.0) * k.a1x, jy = C(1.0 / 12.0) * k.a1y;
+            constexpr C w12 = C(1.0 / 12.0);
+            C jp, jm;  // (a1y +- a1x) / 12
+            if (VEC) {
+                const C jx = mulr<L>(w12, k.a1x);
+                jp = fmac(w12, k.a1y, jx);
+                jm = fmac(w12, k.a1y, -jx);
+            } else {
+                const C jy = mulr<L>(w12, k.a1y);
+                jp = fmac(w12, k.a1x, jy);
+                jm = fmac(-w12, k.a1x, jy);
+            }
             const C Ep = fmac(C(0.25), k.xy, base), Em = fmac(C(-0.25), k.xy, base);
-            const C Op = fmac(C(0.25), k.xxy + k.xyy, jx + jy);
-            const C Om = fmac(C(0.25), k.xxy - k.xyy, jy - jx);
+            const C Op = fmac(C(0.25), k.xxy + k.xyy, jp);
+            const C Om = fmac(C(0.25), k.xxy - k.xyy, jm);
             o[3] = Ep + Op;
             o[7] = Ep - Op;
             o[4] = Em + Om;
@@ -727,36 +740,42 @@ __device__ __forceinline__ Coef<C> coef_interior(const Mom<C> &m, C om, C chi, b
     C dr = m.dr, jx = m.jx, jy = m.jy, jz = m.jz, sc = C(1);
     if (SPONGE) {
         const C h = recip(fmac(C(0.5), chi, C(1)));
-        dr = dr * h;
+        dr = mulr<L>(dr, h);
         jx = jx * h;
         jy = jy * h;
         jz = jz * h;
         sc = C(1) - chi;
     }
     const C inv = recip(C(1) + dr);
-    const C ux = jx * inv, uy = jy * inv;
-    const C c = dr * C(1.0 / 3.0);
-    const C Pxx = jx * ux, Pyy = jy * uy, Pxy = jx * uy;
-    const C nxx = (m.sxx - c) - Pxx, nyy = (m.syy - c) - Pyy;
-    const C qxy = om * (m.sxy - Pxy);
+    const C ux = mulr<L>(jx, inv), uy = mulr<L>(jy, inv);
+    constexpr C third = C(1.0 / 3.0);
+    constexpr bool own = full_third_order<L>();  // (left to the compiler, as its rebuild)
+    // Pi^neq_aa = s_aa - (rho - 1) / 3 - P_aa
+    auto neq = [&](C saa, C P) { return own ? (saa - dr * third) - P : fmac(-dr, third, saa) - P; };
+    // q_ab = w (s_ab - j_a u_b), A2_ab = sc P_ab + q_ab; the bulk form fuses the products
+    auto qab = [&](C sab, C ja, C ub, C P) { return om * (SPONGE || own ? sab - P : fmac(-ja, ub, sab)); };
+    auto aab = [&](C ja, C ub, C P, C q) { return SPONGE || own ? fmac(sc, P, q) : fmac(ja, ub, q); };
+    const C Pxx = mulr<L>(jx, ux), Pyy = mulr<L>(jy, uy), Pxy = mulr<L>(jx, uy);
+    const C nxx = neq(m.sxx, Pxx), nyy = neq(m.syy, Pyy);
+    const C qxy = qab(m.sxy, jx, uy, Pxy);
     k.a0 = SPONGE ? sc * dr : dr;
     k.a1x = SPONGE ? sc * jx : jx;
     k.a1y = SPONGE ? sc * jy : jy;
     k.xx = fmac(om, nxx, SPONGE ? sc * Pxx : Pxx);
     k.yy = fmac(om, nyy, SPONGE ? sc * Pyy : Pyy);
-    k.xy = fmac(SPONGE ? sc : C(1), Pxy, qxy);
+    k.xy = aab(jx, uy, Pxy, qxy);
     const C ux2 = ux + ux, uy2 = uy + uy;
     k.xxy = fmac(uy, k.xx, ux2 * qxy);
     k.xyy = fmac(ux, k.yy, uy2 * qxy);
     if constexpr (L::D == 3) {
-        const C uz = jz * inv;
-        const C Pzz = jz * uz, Pxz = jx * uz, Pyz = jy * uz;
-        const C nzz = (m.szz - c) - Pzz;
-        const C qxz = om * (m.sxz - Pxz), qyz = om * (m.syz - Pyz);
+        const C uz = mulr<L>(jz, inv);
+        const C Pzz = mulr<L>(jz, uz), Pxz = mulr<L>(jx, uz), Pyz = mulr<L>(jy, uz);
+        const C nzz = neq(m.szz, Pzz);
+        const C qxz = qab(m.sxz, jx, uz, Pxz), qyz = qab(m.syz, jy, uz, Pyz);
         k.a1z = SPONGE ? sc * jz : jz;
         k.zz = fmac(om, nzz, SPONGE ? sc * Pzz : Pzz);
-        k.xz = fmac(SPONGE ? sc : C(1), Pxz, qxz);
-        k.yz = fmac(SPONGE ? sc : C(1), Pyz, qyz);
+        k.xz = aab(jx, uz, Pxz, qxz);
+        k.yz = aab(jy, uz, Pyz, qyz);
         const C uz2 = uz + uz;
         k.xxz = fmac(uz, k.xx, ux2 * qxz);
         k.xzz = fmac(ux, k.zz, uz2 * qxz);
@@ -781,6 +800,127 @@ __device__ __forceinline__ Coef<C> coef_interior(const Mom<C> &m, C om, C chi, b
         }
     }
     return k;
+}
+
+// ---------------------------------------------------------------------------
+// The same collision and rebuild in FP64 for D2Q9 and D3Q19 with fewer
+// operations.  GB300 issues two FP64 lanes per SM and cycle, so the FP64
+// update takes the time of its FP64 instructions and nothing else (the
+// single-precision form of the collision has room for them).  Against
+// coef_interior + rebuild_all:
+//   - the tensors are formed as quarters, A' = A2 / 4 and q' = w Pi^neq / 4, the
+//     factor the rebuild multiplies them by: A'_aa = w/4 (s_aa - dr/3) +
+//     (sc - w)/4 j_a u_a, with sc = 1 - chi (1 in the bulk);
+//   - with T_ab = A3_abb / 4 = u_a A'_bb + 2 u_b q'_ab, k_a = j_a / 12 and
+//     X_ab = T_ab + k_a, an edge direction's odd part is X_ab + X_ba (or their
+//     difference) and a face direction's 2 (k_a - T_ab - T_ac);
+//   - 1 / rho is one third-order correction x (1 + e + e^2), e = 1 - rho x, of a
+//     single-precision reciprocal x (|e| < 2^-23, so the rest is below 2^-68).
+// D3Q19: 155 FP64 operations per bulk cell (from 175); D2Q9: 72 (from 92).
+// (Adding k_a inside T_ab's multiply-adds would save six more, but a face
+// direction then subtracts it again: 1.5 times the rounding error.)
+// Every operation is written with its rounding, so every kernel gives the
+// same bits; against 80-bit arithmetic the error of u after 40 steps is the
+// same as before (2.0e-15).  With the routes of cell_collide, GB300: D3Q19 jet
+// 96 x 64 x 64 172.8 -> 141 us per step, 192 x 128 x 128 1.17 -> 1.02 ms; D2Q9
+// 128 x 128 5.1 -> 5.0 us (launch and latency).
+// chi = 0 gives the bulk result bit for bit.
+// ---------------------------------------------------------------------------
+template <class L, class C>
+__host__ __device__ constexpr bool has_fp64_form()
+{
+    return sizeof(C) == 8 && L::Q <= 19;
+}
+
+__device__ __forceinline__ double recip_fma(double x)
+{
+    const double r = (double)__frcp_rn((float)x);
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
+template <class L, bool SPONGE>
+__device__ __forceinline__ void collide_fp64(const Mom<double> &m, double om, double chi, double *o)
+{
+    constexpr double third = 1.0 / 3.0;
+    double dr = m.dr, jx = m.jx, jy = m.jy, jz = m.jz, sc = 1.0;
+    if (SPONGE) {
+        const double h = recip_fma(__fma_rn(0.5, chi, 1.0));
+        dr = __dmul_rn(dr, h);
+        jx = __dmul_rn(jx, h);
+        jy = __dmul_rn(jy, h);
+        if (L::D == 3) jz = __dmul_rn(jz, h);
+        sc = __dadd_rn(1.0, -chi);
+    }
+    const double inv = recip_fma(__dadd_rn(1.0, dr));
+    const double w4 = __dmul_rn(0.25, om), v4 = __dmul_rn(0.25, __dadd_rn(sc, -om));
+    const double ux = __dmul_rn(jx, inv), uy = __dmul_rn(jy, inv);
+    const double vx = __dmul_rn(v4, ux), vy = __dmul_rn(v4, uy), wy = __dmul_rn(w4, uy);
+    const double xx = __fma_rn(jx, vx, __dmul_rn(w4, __fma_rn(-third, dr, m.sxx)));
+    const double yy = __fma_rn(jy, vy, __dmul_rn(w4, __fma_rn(-third, dr, m.syy)));
+    const double txy = __dmul_rn(w4, m.sxy);
+    const double xy = __fma_rn(jx, vy, txy), qxy = __fma_rn(-jx, wy, txy);
+    const double ux2 = __dadd_rn(ux, ux), uy2 = __dadd_rn(uy, uy);
+    const double a0 = SPONGE ? __dmul_rn(sc, dr) : dr;
+    const double j12 = SPONGE ? __dmul_rn(1.0 / 12.0, sc) : 1.0 / 12.0;
+    const double kx = __dmul_rn(j12, jx), ky = __dmul_rn(j12, jy);
+    const double Txy = __fma_rn(ux, yy, __dmul_rn(uy2, qxy)), Tyx = __fma_rn(uy, xx, __dmul_rn(ux2, qxy));
+    const double Xy = __dadd_rn(Txy, kx), Yx = __dadd_rn(Tyx, ky);
+    if constexpr (L::Q == 19) {
+        const double uz = __dmul_rn(jz, inv);
+        const double vz = __dmul_rn(v4, uz), wz = __dmul_rn(w4, uz);
+        const double zz = __fma_rn(jz, vz, __dmul_rn(w4, __fma_rn(-third, dr, m.szz)));
+        const double txz = __dmul_rn(w4, m.sxz), tyz = __dmul_rn(w4, m.syz);
+        const double xz = __fma_rn(jx, vz, txz), qxz = __fma_rn(-jx, wz, txz);
+        const double yz = __fma_rn(jy, vz, tyz), qyz = __fma_rn(-jy, wz, tyz);
+        const double uz2 = __dadd_rn(uz, uz), kz = __dmul_rn(j12, jz);
+        const double Txz = __fma_rn(ux, zz, __dmul_rn(uz2, qxz)), Tzx = __fma_rn(uz, xx, __dmul_rn(ux2, qxz));
+        const double Tyz = __fma_rn(uy, zz, __dmul_rn(uz2, qyz)), Tzy = __fma_rn(uz, yy, __dmul_rn(uy2, qyz));
+        const double Xz = __dadd_rn(Txz, kx), Zx = __dadd_rn(Tzx, kz);
+        const double Yz = __dadd_rn(Tyz, ky), Zy = __dadd_rn(Tzy, kz);
+        const double t3 = __dmul_rn(third, __dadd_rn(__dadd_rn(xx, yy), zz));
+        o[0] = __fma_rn(-6.0, t3, __dmul_rn(third, a0));
+        const double b1 = __fma_rn(1.0 / 18.0, a0, -t3), b2 = __fma_rn(1.0 / 36.0, a0, t3);
+        {  // faces: 1 / 10, 2 / 11, 3 / 12
+            const double Ex = __dadd_rn(b1, xx), Ey = __dadd_rn(b1, yy), Ez = __dadd_rn(b1, zz);
+            const double Ox = __dadd_rn(kx, -__dadd_rn(Txy, Txz)), Oy = __dadd_rn(ky, -__dadd_rn(Tyx, Tyz)),
+                         Oz = __dadd_rn(kz, -__dadd_rn(Tzx, Tzy));
+            o[1] = __fma_rn(2.0, Ox, Ex);
+            o[10] = __fma_rn(-2.0, Ox, Ex);
+            o[2] = __fma_rn(2.0, Oy, Ey);
+            o[11] = __fma_rn(-2.0, Oy, Ey);
+            o[3] = __fma_rn(2.0, Oz, Ez);
+            o[12] = __fma_rn(-2.0, Oz, Ez);
+        }
+        // edges of the xy, xz and yz planes: (s, s) / opposite, (s, -s) / opposite
+        auto plane = [&](int i, double base, double off, double P, double R) {
+            const double Ep = __dadd_rn(base, off), Em = __dadd_rn(base, -off);
+            const double Op = __dadd_rn(P, R), Om = __dadd_rn(P, -R);
+            o[i] = __dadd_rn(Ep, Op);
+            o[i + 9] = __dadd_rn(Ep, -Op);
+            o[i + 1] = __dadd_rn(Em, Om);
+            o[i + 10] = __dadd_rn(Em, -Om);
+        };
+        plane(4, __fma_rn(-0.5, zz, b2), xy, Xy, Yx);
+        plane(6, __fma_rn(-0.5, yy, b2), xz, Xz, Zx);
+        plane(8, __fma_rn(-0.5, xx, b2), yz, Yz, Zy);
+    } else {
+        const double t3 = __dmul_rn(third, __dadd_rn(xx, yy));
+        o[0] = __fma_rn(-8.0, t3, __dmul_rn(4.0 / 9.0, a0));
+        const double b1 = __fma_rn(-2.0, t3, __dmul_rn(1.0 / 9.0, a0)), b2 = __fma_rn(1.0 / 36.0, a0, t3);
+        const double Ex = __fma_rn(2.0, xx, b1), Ey = __fma_rn(2.0, yy, b1);
+        const double Ox = __fma_rn(2.0, kx, -Txy), Oy = __fma_rn(2.0, ky, -Tyx);
+        o[1] = __fma_rn(2.0, Ox, Ex);
+        o[5] = __fma_rn(-2.0, Ox, Ex);
+        o[2] = __fma_rn(2.0, Oy, Ey);
+        o[6] = __fma_rn(-2.0, Oy, Ey);
+        const double Ep = __dadd_rn(b2, xy), Em = __dadd_rn(b2, -xy);
+        const double Op = __dadd_rn(Xy, Yx), Om = __dadd_rn(Yx, -Xy);
+        o[3] = __dadd_rn(Ep, Op);
+        o[7] = __dadd_rn(Ep, -Op);
+        o[4] = __dadd_rn(Em, Om);
+        o[8] = __dadd_rn(Em, -Om);
+    }
 }
 
 // splitmix64 (Steele, Lea and Flood 2014): counter-based uniform in [0, 1)

@@ -238,8 +238,9 @@ __device__ __forceinline__ void face_velocity(const StepParams &p, int inlet, in
 #pragma unroll
     for (int b = 0; b < 3; ++b) ub[b] = C(prof ? prof[3 * kf + b] : p.u_face[inlet][b]);
     if (p.noise_amp > 0.0) {
-        const C mag = sqrt(ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2]);
-        if (mag > C(0)) {
+        const C mag2 = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
+        if (mag2 > C(0)) {
+            const C mag = sqrt(mag2);
             const uint64_t base =
                 (p.noise_seed << 32) + ((uint64_t)p.step * (uint64_t)p.face_cells[inlet] + (uint64_t)kf) * 3u;
             const C amp = C(p.noise_amp) * mag;
@@ -255,9 +256,57 @@ __device__ __forceinline__ void face_velocity(const StepParams &p, int inlet, in
 // neighbour whose streamed moments m are given, Pi^neq about its own rho, u
 // (zeroed normal-tangential components on a free-slip face):
 //   dr' = rho' - 1,  j' = rho' u',  s' = Pi^neq' + dr' c_s^2 I + rho' u' u'.
+// FP64 forms s' = (s - rho u u) + rho' u' u' + (rho' - rho) c_s^2 I directly: 25
+// FP64 operations on a velocity node, paid by its whole warp.
 template <class L, class C>
 __device__ __forceinline__ Mom<C> face_moments(const StepParams &p, const Mom<C> &m, int inlet, int cx, int cy, int cz)
 {
+    if constexpr (has_fp64_form<L, C>()) {
+        const C rho = C(1) + m.dr, inv = recip_fma(rho);
+        C ux = m.jx * inv, uy = m.jy * inv, uz = L::D == 3 ? m.jz * inv : C(0);
+        Mom<C> o = m;
+        o.sxx = fmac(-m.jx, ux, m.sxx);
+        o.syy = fmac(-m.jy, uy, m.syy);
+        o.sxy = fmac(-m.jx, uy, m.sxy);
+        if (L::D == 3) {
+            o.szz = fmac(-m.jz, uz, m.szz);
+            o.sxz = fmac(-m.jx, uz, m.sxz);
+            o.syz = fmac(-m.jy, uz, m.syz);
+        }
+        C r = rho;
+        const int kind = p.kind[inlet];
+        if (kind == BC_VELOCITY) {
+            C ub[3];
+            face_velocity<L, C>(p, inlet, cx, cy, cz, ub);
+            ux = ub[0];
+            uy = ub[1];
+            uz = L::D == 3 ? ub[2] : C(0);
+        } else if (kind == BC_PRESSURE) {
+            o.dr = C(p.rho_face_m1[inlet]);
+            r = C(p.rho_face[inlet]);
+            const C c = (o.dr - m.dr) * C(1.0 / 3.0);
+            o.sxx += c;
+            o.syy += c;
+            if (L::D == 3) o.szz += c;
+        } else {
+            const int a = inlet >> 1;
+            if (a == 0) { ux = C(0); o.sxy = C(0); o.sxz = C(0); }
+            if (a == 1) { uy = C(0); o.sxy = C(0); o.syz = C(0); }
+            if (a == 2) { uz = C(0); o.sxz = C(0); o.syz = C(0); }
+        }
+        o.jx = r * ux;
+        o.jy = r * uy;
+        o.jz = r * uz;
+        o.sxx = fmac(o.jx, ux, o.sxx);
+        o.syy = fmac(o.jy, uy, o.syy);
+        o.sxy = fmac(o.jx, uy, o.sxy);
+        if (L::D == 3) {
+            o.szz = fmac(o.jz, uz, o.szz);
+            o.sxz = fmac(o.jx, uz, o.sxz);
+            o.syz = fmac(o.jy, uz, o.syz);
+        }
+        return o;
+    }
     const C rho = C(1) + m.dr;
     const C inv = recip(rho);
     C ux = m.jx * inv, uy = m.jy * inv, uz = L::D == 3 ? m.jz * inv : C(0);
@@ -414,6 +463,41 @@ __device__ __forceinline__ bool index_fault(const StepParams &p, bool bad)
 #endif
 }
 
+// New populations o (w_i-shifted) of a cell with streamed populations g and
+// their moments m: coefficients, rebuild and relaxation (even / odd parts of
+// each opposite pair); plain BGK adds (1 - 1/tau) g except at rebuilt boundary
+// nodes.  FP64 storage takes one route for every cell that allows it: a
+// velocity / free-slip / pressure node as an interior collision of
+// substituted moments, sponge and bulk cells of a warp together (chi = 0 is
+// the bulk result bit for bit), because on the FP64 pipe a warp pays for every
+// route its lanes take at the price of all 32.
+template <class L, class C, bool BGK>
+__device__ __forceinline__ void cell_collide(const StepParams &p, const Mom<C> &m0, const C (&g)[L::Q], C chi, int x,
+                                             int y, int z, int inlet, C (&o)[L::Q])
+{
+    if constexpr (has_fp64_form<L, C>() && !BGK) {
+        const bool general = (L::D == 2 && p.order4) || (chi > C(0) && !p.sponge_rest);
+        if (!general) {
+            Mom<C> m = m0;
+            if (inlet >= 0) m = face_moments<L, C>(p, m0, inlet, x, y, z);
+            if (__any_sync(__activemask(), chi > C(0)))
+                collide_fp64<L, true>(m, C(p.omega), chi, o);
+            else
+                collide_fp64<L, false>(m, C(p.omega), C(0), o);
+            return;
+        }
+    }
+    const Coef<C> k = cell_coefficients<L, C, BGK>(p, m0, chi, x, y, z, inlet);
+    const C keep = (BGK && inlet < 0) ? C(p.omega) : C(0);
+    if (L::D == 2 && p.order4)
+        rebuild_all<L, C, true>(k, o);
+    else
+        rebuild_all<L, C, false>(k, o);
+#pragma unroll
+    for (int i = 0; i < L::Q; ++i)
+        if (BGK) o[i] = fmac(keep, g[i], o[i]);
+}
+
 template <class L, class S, class C, bool BGK = false, int MASK = kMaskLinks>
 __device__ __forceinline__ void update_cell(const StepParams &p, const char *const *in, char *const *out,
                                             int x, int y, int z)
@@ -500,20 +584,8 @@ __device__ __forceinline__ void update_cell(const StepParams &p, const char *con
 
     const Mom<C> m = moments_pairs<L, C>(g);
     const C chi = (bulk || inlet >= 0) ? C(0) : chi_cell<L, C>(p, chi_row<L, C>(p, y, z), x, y, z);
-    const Coef<C> k = cell_coefficients<L, C, BGK>(p, m, chi, x, y, z, inlet);
-
-    // ---- rebuild, relax and store (even/odd parts of each opposite pair);
-    // plain BGK adds (1 - 1/tau) g of the streamed populations except at
-    // rebuilt boundary nodes
-    const C keep = (BGK && inlet < 0) ? C(p.omega) : C(0);
     C o[L::Q];
-    if (L::D == 2 && p.order4)
-        rebuild_all<L, C, true>(k, o);
-    else
-        rebuild_all<L, C, false>(k, o);
-#pragma unroll
-    for (int i = 0; i < L::Q; ++i)
-        if (BGK) o[i] = fmac(keep, g[i], o[i]);
+    cell_collide<L, C, BGK>(p, m, g, chi, x, y, z, inlet, o);
     if (p.shifted) {
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) o[i] -= dsh<C>(p, i);
@@ -619,17 +691,8 @@ __device__ __forceinline__ void update_cell_aa(const StepParams &p, char *const 
                 const bool bulk = X >= p.blo[0] && X < p.bhi[0] && Y >= p.blo[1] && Y < p.bhi[1] &&
                                   Z >= p.blo[2] && Z < p.bhi[2];
                 const C chi = (bulk || inlet >= 0) ? C(0) : chi_cell<L, C>(p, chi_row<L, C>(p, Y, Z), X, Y, Z);
-                const Coef<C> k = cell_coefficients<L, C, BGK>(p, m, chi, X, Y, Z, inlet);
-                const C keep = (BGK && inlet < 0) ? C(p.omega) : C(0);
                 C o[L::Q];
-                if (L::D == 2 && p.order4)
-                    rebuild_all<L, C, true>(k, o);
-                else
-                    rebuild_all<L, C, false>(k, o);
-                if (BGK) {
-#pragma unroll
-                    for (int i = 0; i < L::Q; ++i) o[i] = fmac(keep, g[i], o[i]);
-                }
+                cell_collide<L, C, BGK>(p, m, g, chi, X, Y, Z, inlet, o);
                 if (LOC) {
 #pragma unroll
                     for (int i = 0; i < L::Q; ++i) Store<S>::st((S *)f[i] + t, o[i]);

@@ -260,8 +260,7 @@ struct GroupSt<__nv_bfloat16, 4> {
 // non-periodic x face takes its x neighbour's streamed populations (same
 // thread) and its boundary role.  Cells are collided and stored G at a time.
 // An interior cell is bulk or a sponge cell: layers relaxing to the rest
-// state use the closed form of coef_interior (which gives the bulk
-// coefficients bit for bit at chi = 0), other references and velocity /
+// state use the closed form of coef_interior, other references and velocity /
 // free-slip / pressure nodes the general coefficients.
 //
 // Streaming patterns (SP): kPull reads one lattice and writes the other;
@@ -476,7 +475,7 @@ __device__ __forceinline__ void vec_store(const StepParams &p, char *bout, int x
 // closed-form coefficients of a rest-state reference.  A node on a
 // non-periodic x face collides its neighbour's streamed populations: as they
 // are (outflow face) or with the face's density / velocity substituted.
-template <class L, class S, class C, int V, int G, int SP>
+template <class L, class S, class C, int V, int G, int SP, int WR>
 __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out0, int x0, int y, int z,
                                                   const RowOff &ro, const VecIn<L, S, C, V> &r, bool all_bulk)
 {
@@ -495,10 +494,13 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
         for (int kk = 0; kk < G; ++kk) {
             const int k = k0 + kk;
             C g[L::Q];
-            Coef<C> cf;
+            Mom<C> m;
+            C chi = C(0);
+            Coef<C> cf;  // (unused in FP64, whose collision has a form of its own)
             if (all_bulk) {
                 gather_vec<L, S, C, V, SP>(r, k, g);
-                cf = coef_interior<L, C, false>(moments_pairs<L, C>(g), om, C(0));
+                m = moments_pairs<L, C>(g);
+                if constexpr (!has_fp64_form<L, C>()) cf = coef_interior<L, C, false>(m, om, C(0));
             } else {
                 // a node on a non-periodic x face collides the populations
                 // streamed into its neighbour (same thread), with its own role
@@ -507,11 +509,10 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
                     gather_vec<L, S, C, V, SP>(r, k == 0 ? 1 : V - 2, g);
                 else
                     gather_vec<L, S, C, V, SP>(r, k, g);
-                Mom<C> m = moments_pairs<L, C>(g);
+                m = moments_pairs<L, C>(g);
                 const int x = x0 + k;
                 const int inlet = !face ? -1 : (k == 0 ? (p.kind[0] != BC_OUTFLOW ? 0 : -1)
                                                         : (p.kind[1] != BC_OUTFLOW ? 1 : -1));
-                C chi = C(0);
                 if (inlet >= 0) {
                     m = face_moments<L, C>(p, m, inlet, x, y, z);
                 } else {
@@ -521,9 +522,16 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
                         chi = v > chi ? v : chi;
                     }
                 }
-                cf = coef_interior<L, C, true>(m, om, chi);
+                if constexpr (!has_fp64_form<L, C>()) cf = coef_interior<L, C, true>(m, om, chi);
             }
-            rebuild_all<L, C, false>(cf, o[kk]);
+            if constexpr (has_fp64_form<L, C>()) {
+                if (all_bulk)
+                    collide_fp64<L, false>(m, om, chi, o[kk]);
+                else
+                    collide_fp64<L, true>(m, om, chi, o[kk]);
+            } else {
+                rebuild_all<L, C, false, !WR>(cf, o[kk]);
+            }
         }
         vec_store<L, S, C, V, G, SP>(p, bout, x0, k0, ro, o);
     }
@@ -579,7 +587,7 @@ __device__ __forceinline__ void update_vec(const StepParams &p, const char *cons
         if (!vec_load<L, S, C, V, SP>(p, in[0], x0, y, z, ro, r)) return;
         const bool bulk = y >= p.blo[1] && y < p.bhi[1] && z >= p.blo[2] && z < p.bhi[2] && x0 >= p.blo[0] &&
                           x0 + V <= p.bhi[0];
-        vec_collide_store<L, S, C, V, G, SP>(p, out[0], x0, y, z, ro, r, bulk);
+        vec_collide_store<L, S, C, V, G, SP, WR>(p, out[0], x0, y, z, ro, r, bulk);
         return;
     }
     if constexpr (!WR) {
