@@ -29,6 +29,9 @@
 #include <deque>
 #include <map>
 #include <string>
+#include <system_error>
+#include <thread>
+#include <utility>
 #include <vector>
 
 #include "lbm.h"
@@ -50,10 +53,13 @@ struct Request {
     size_t bytes = 0;
     int state = LBM_REQ_QUEUED;
     int slot = -1;
-    std::vector<double> rho, u;      // initial state, then the result
+    // initial state, then the result: rho (ncell), u (3 ncell).  Page-locked from
+    // the server's pool, read and written by the GPU directly, or (beyond the
+    // pool's bound, while queued) pageable
+    double *host = nullptr;
+    std::vector<double> pageable;
     void *f[2] = {nullptr, nullptr};
     bool aa = false;                 // one lattice, in-place AA steps
-    double *res_h = nullptr;         // pinned result: rho (ncell), then u (3 ncell)
     cudaEvent_t res_ev = nullptr;    // recorded behind the result copy
     bool retiring = false;           // result copy enqueued, not yet finalised
 };
@@ -205,8 +211,82 @@ struct lbm_server {
     double gpu_ms = 0.0;
     int64_t rounds = 0;
     std::vector<Request *> retiring;     // results in flight
+    std::vector<std::pair<double *, size_t>> blocks;  // page-locked blocks kept for reuse
+    std::map<double *, size_t> held;     // blocks in use by requests
+    size_t kept = 0, held_bytes = 0;
     std::string err;
 };
+
+// Page-locked host blocks.  Allocating and freeing one per request cost more
+// than its copies: the blocks of finished requests are kept for the next ones,
+// at most kPinnedKept bytes of them, and given back when the server is
+// destroyed.  Queued requests hold at most kPinnedMax bytes of blocks.
+constexpr size_t kPinnedKept = size_t(256) << 20, kPinnedMax = size_t(1) << 30;
+
+static size_t host_bytes(const Request *r) { return sizeof(double) * 4 * (size_t)r->ncell; }
+
+// A block of at least `bytes` (null: allocation failed)
+static double *take_block(lbm_server *s, size_t bytes)
+{
+    auto best = s->blocks.end();
+    for (auto it = s->blocks.begin(); it != s->blocks.end(); ++it)
+        if (it->second >= bytes && it->second <= 2 * bytes && (best == s->blocks.end() || it->second < best->second))
+            best = it;
+    double *b = nullptr;
+    size_t size = bytes;
+    if (best != s->blocks.end()) {
+        b = best->first;
+        size = best->second;
+        s->kept -= size;
+        s->blocks.erase(best);
+    } else if (cudaHostAlloc((void **)&b, bytes, cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    s->held[b] = size;
+    s->held_bytes += size;
+    return b;
+}
+
+// Give a block back (its last use by the GPU has completed)
+static void return_block(lbm_server *s, double *b)
+{
+    if (!b) return;
+    auto it = s->held.find(b);
+    const size_t size = it->second;
+    s->held.erase(it);
+    s->held_bytes -= size;
+    if (s->kept + size > kPinnedKept) {
+        cudaFreeHost(b);
+        return;
+    }
+    s->blocks.emplace_back(b, size);
+    s->kept += size;
+}
+
+// Copy between host buffers; large ones by four threads (one core's copy rate
+// is a fraction of the memory's)
+static void copy_host(double *dst, const double *src, size_t n)
+{
+    constexpr size_t kPart = size_t(1) << 18;  // doubles a thread is worth starting for
+    const size_t parts = std::min<size_t>(4, n / kPart);
+    if (parts < 2) {
+        std::memcpy(dst, src, n * sizeof(double));
+        return;
+    }
+    std::vector<std::thread> th;
+    try {
+        for (size_t k = 1; k < parts; ++k) {
+            const size_t a = n * k / parts, b = n * (k + 1) / parts;
+            th.emplace_back([=] { std::memcpy(dst + a, src + a, (b - a) * sizeof(double)); });
+        }
+    } catch (const std::system_error &) {  // no thread to be had: the rest here
+        const size_t a = n * (th.size() + 1) / parts;
+        std::memcpy(dst + a, src + a, (n - a) * sizeof(double));
+    }
+    std::memcpy(dst, src, n / parts * sizeof(double));
+    for (std::thread &t : th) t.join();
+}
 
 static int sfail(lbm_server *s, int code, const char *fmt, ...)
 {
@@ -274,11 +354,11 @@ static void free_request_memory(lbm_server *s, Request *r)
     r->f[0] = r->f[1] = nullptr;
 }
 
-static void free_request_host(Request *r)
+static void free_request_host(lbm_server *s, Request *r)
 {
-    if (r->res_h) cudaFreeHost(r->res_h);
+    return_block(s, r->host);
     if (r->res_ev) cudaEventDestroy(r->res_ev);
-    r->res_h = nullptr;
+    r->host = nullptr;
     r->res_ev = nullptr;
 }
 
@@ -288,7 +368,7 @@ extern "C" void lbm_server_destroy(lbm_server_handle s)
     cudaStreamSynchronize(s->stream);
     for (auto &kv : s->reqs) {
         free_request_memory(s, kv.second);
-        free_request_host(kv.second);
+        free_request_host(s, kv.second);
         delete kv.second;
     }
     cudaStreamSynchronize(s->stream);
@@ -297,6 +377,7 @@ extern "C" void lbm_server_destroy(lbm_server_handle s)
         if (s->gpu_t0[k]) cudaEventDestroy(s->gpu_t0[k]);
         if (s->gpu_t1[k]) cudaEventDestroy(s->gpu_t1[k]);
     }
+    for (auto &b : s->blocks) cudaFreeHost(b.first);
     if (s->graph) cudaGraphExecDestroy(s->graph);
     for (int g = 0; g < NGROUPS; ++g) {
         if (s->tiles_d[g]) cudaFree(s->tiles_d[g]);
@@ -340,10 +421,18 @@ extern "C" int lbm_server_submit(lbm_server_handle s, const lbm_request *req, in
         delete r;
         return sfail(s, LBM_EINVAL, "request needs %zu bytes, more than the whole budget (%zu)", need, s->budget);
     }
-    r->rho.assign((size_t)r->ncell, 1.0);
-    r->u.assign((size_t)r->ncell * 3, 0.0);
-    if (req->rho) std::memcpy(r->rho.data(), req->rho, sizeof(double) * (size_t)r->ncell);
-    if (req->u) std::memcpy(r->u.data(), req->u, sizeof(double) * 3 * (size_t)r->ncell);
+    const size_t N = (size_t)r->ncell;
+    if (s->held_bytes + host_bytes(r) <= kPinnedMax) r->host = take_block(s, host_bytes(r));
+    if (!r->host) r->pageable.resize(4 * N);
+    double *h = r->host ? r->host : r->pageable.data();
+    if (req->rho)
+        copy_host(h, req->rho, N);
+    else
+        std::fill(h, h + N, 1.0);
+    if (req->u)
+        copy_host(h + N, req->u, 3 * N);
+    else
+        std::fill(h + N, h + 4 * N, 0.0);
     r->id = s->next_id++;
     s->reqs[r->id] = r;
     s->queue.push_back(r);
@@ -384,18 +473,19 @@ static int admit(lbm_server *s)
             ++it;  // device memory short of the budget: try again next round
             continue;
         }
-        double *buf = nullptr;
-        e = cudaMallocAsync((void **)&buf, sizeof(double) * 4 * (size_t)r->ncell, s->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(buf, r->rho.data(), sizeof(double) * (size_t)r->ncell, cudaMemcpyHostToDevice, s->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(buf + r->ncell, r->u.data(), sizeof(double) * 3 * (size_t)r->ncell,
-                                cudaMemcpyHostToDevice, s->stream);
-        if (e == cudaSuccess) e = TYPED(init_eq, r->lattice, r->prec, *r, buf, buf + r->ncell, s->stream);
-        if (buf) cudaFreeAsync(buf, s->stream);
+        if (r->host) {
+            // the kernel reads the page-locked block over the host link
+            e = TYPED(init_eq, r->lattice, r->prec, *r, r->host, r->host + r->ncell, s->stream);
+        } else {
+            double *buf = nullptr;
+            e = cudaMallocAsync((void **)&buf, host_bytes(r), s->stream);
+            if (e == cudaSuccess)  // (pageable: staged by the call)
+                e = cudaMemcpyAsync(buf, r->pageable.data(), host_bytes(r), cudaMemcpyHostToDevice, s->stream);
+            if (e == cudaSuccess) e = TYPED(init_eq, r->lattice, r->prec, *r, buf, buf + r->ncell, s->stream);
+            if (buf) cudaFreeAsync(buf, s->stream);
+            std::vector<double>().swap(r->pageable);
+        }
         if (e != cudaSuccess) return sfail(s, LBM_ECUDA, "admitting request %lld: %s", (long long)r->id, cudaGetErrorString(e));
-        std::vector<double>().swap(r->rho);
-        std::vector<double>().swap(r->u);
         BatchDomain d{};
         std::memset(&d, 0, sizeof d);
         for (int a = 0; a < 3; ++a) {
@@ -542,14 +632,13 @@ static int retire_slot(lbm_server *s, int k)
     const int par = (int)(r->steps & 1);  // lattice (pull) / layout (AA) after the last step
     cudaError_t e = cudaSuccess;
     if (r->aa && par) e = TYPED(unswap, r->lattice, r->prec, *r, s->doms_h[k].p, s->stream);
-    double *buf = nullptr;
-    if (e == cudaSuccess) e = cudaMallocAsync((void **)&buf, sizeof(double) * 4 * (size_t)r->ncell, s->stream);
-    if (e == cudaSuccess) e = TYPED(moments, r->lattice, r->prec, *r, r->aa ? 0 : par, buf, buf + r->ncell, s->stream);
-    if (e == cudaSuccess && !r->res_h)
-        e = cudaHostAlloc((void **)&r->res_h, sizeof(double) * 4 * (size_t)r->ncell, cudaHostAllocDefault);
+    if (e == cudaSuccess && !r->host) {
+        r->host = take_block(s, host_bytes(r));
+        if (!r->host) e = cudaErrorMemoryAllocation;
+    }
+    // the kernel writes the page-locked block over the host link
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(r->res_h, buf, sizeof(double) * 4 * (size_t)r->ncell, cudaMemcpyDeviceToHost, s->stream);
-    if (buf) cudaFreeAsync(buf, s->stream);
+        e = TYPED(moments, r->lattice, r->prec, *r, r->aa ? 0 : par, r->host, r->host + r->ncell, s->stream);
     if (e == cudaSuccess && !r->res_ev) e = cudaEventCreateWithFlags(&r->res_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(r->res_ev, s->stream);
     if (e != cudaSuccess) return sfail(s, LBM_ECUDA, "retiring request %lld: %s", (long long)r->id, cudaGetErrorString(e));
@@ -573,8 +662,15 @@ static int finalize(lbm_server *s, Request *r, bool wait, bool *finished)
     const cudaError_t q = wait ? cudaEventSynchronize(r->res_ev) : cudaEventQuery(r->res_ev);
     if (q == cudaErrorNotReady) return LBM_OK;
     if (q != cudaSuccess) return sfail(s, LBM_ECUDA, "result of request %lld: %s", (long long)r->id, cudaGetErrorString(q));
-    bool finite = true;
-    for (int64_t c = 0; c < r->ncell; ++c) finite = finite && std::isfinite(r->res_h[c]);
+    // rho finite everywhere: no exponent of all ones (without a branch per value)
+    constexpr uint64_t kExp = 0x7ff0000000000000ull;
+    uint64_t bad = 0;
+    for (int64_t c = 0; c < r->ncell; ++c) {
+        uint64_t v;
+        std::memcpy(&v, r->host + c, sizeof v);
+        bad += (v & kExp) == kExp ? 1 : 0;
+    }
+    const bool finite = bad == 0;
     r->state = finite ? LBM_REQ_DONE : LBM_REQ_FAILED;
     r->retiring = false;
     s->retiring.erase(std::find(s->retiring.begin(), s->retiring.end(), r));
@@ -731,10 +827,10 @@ extern "C" int lbm_server_result(lbm_server_handle s, int64_t id, double *rho, d
     if (rc0 != LBM_OK) return rc0;
     if (r->state != LBM_REQ_DONE && r->state != LBM_REQ_FAILED)
         return sfail(s, LBM_EINVAL, "request %lld has not finished", (long long)id);
-    if (rho) std::memcpy(rho, r->res_h, sizeof(double) * (size_t)r->ncell);
-    if (u) std::memcpy(u, r->res_h + r->ncell, sizeof(double) * 3 * (size_t)r->ncell);
+    if (rho) copy_host(rho, r->host, (size_t)r->ncell);
+    if (u) copy_host(u, r->host + r->ncell, 3 * (size_t)r->ncell);
     const int st = r->state;
-    free_request_host(r);
+    free_request_host(s, r);
     s->reqs.erase(it);
     delete r;
     return st == LBM_REQ_DONE ? LBM_OK : sfail(s, LBM_EUNSTABLE, "request %lld produced non-finite values", (long long)id);
