@@ -291,12 +291,15 @@ int lbm_probe(lbm_handle h, int n, const int64_t *cells, double *p_prime);
  *   cells_per_thread : 1 = one cell per thread (the general kernel); 2 or 4 =
  *                      vectorised kernel with that many consecutive x cells per
  *                      thread (FP64: 2; FP32, FP16, BF16: 2 or 4); 0 = default
- *                      (measured fastest on GB300: 2 for FP16 / BF16 on D3Q19
- *                      and D3Q27 and for FP32 on D3Q27, else 1).  The
- *                      vectorised kernel is used only when
- *                      there is no cell-type mask and nx is a multiple of it
- *                      (on D3Q27 only with 2 cells per thread); otherwise the
- *                      general kernel runs.  These kernels
+ *                      (measured fastest on GB300: 1 for FP64 and for FP32
+ *                      on D3Q19, else 2).  The vectorised kernel is used only
+ *                      when nx is a multiple of it (on D3Q27 only with 2 cells
+ *                      per thread), a direction's arrays span less than 2 GB in
+ *                      all, and there is no cell-type mask, fourth order or
+ *                      sponge other than face layers relaxing to the rest
+ *                      state; with a storage shift only with 2 cells per thread
+ *                      of 16-bit storage or D2Q9 FP32.  Otherwise the general
+ *                      kernel runs.  These kernels
  *                      run when the row-staged kernel (lbm_set_staging) is off
  *                      or not eligible.
  * lbm_get_launch reports the shape lbm_step will use now.
@@ -419,8 +422,8 @@ int lbm_get_staging(lbm_handle h, int *active, int *stages, int *block, int *row
  * stored field (both lattices) is re-expressed in the new shift on the
  * device.  The arithmetic is unchanged: a loaded value gets
  * feqH_i(1, u_s) - w_i added, a stored one subtracted.  Runs on the general
- * update kernel (the vectorised and row-staged kernels are not used); not with
- * the AA pattern or refinement patches (LBM_EINVAL); |u_s| < c_s.
+ * update kernel or, with 2 cells per thread, the vectorised one (not the
+ * row-staged one); not with the AA pattern or refinement patches (LBM_EINVAL); |u_s| < c_s.
  * Checkpoints record the shift and load only into a handle with the same one.
  */
 int lbm_set_storage_shift(lbm_handle h, const double u_s[3]);

@@ -1,6 +1,7 @@
 // dispatch.h -- entry points of the per-lattice kernel translation units.
 #pragma once
 #include <cuda_runtime.h>
+#include <cstddef>
 #include <cstdint>
 
 namespace rr {
@@ -55,14 +56,22 @@ inline bool vec_supported(int precision, int vec)
     }
     return false;
 }
+// Whether the vectorised pull takes a storage shift: two cells per thread of
+// 16-bit storage, where the shift is for, and of D2Q9 FP32
+constexpr bool vec_shift_supported(int q, size_t elem, int vec)
+{
+    return vec == 2 && (elem == 2 || (elem == 4 && q == 9));
+}
 // Default cells per thread, measured on GB300 (round jet 384 x 256 x 256,
 // G cell updates/s, one cell per thread vs two): D3Q19 FP16 52.9 vs 63.2,
 // FP64 2.05 vs 2.00, FP32 at the copy bandwidth either way; D3Q27 FP32 31.4
-// vs 32.4, FP16 38.0 vs 44.5; D2Q9 (1600 x 800) FP32 89 vs 81, FP16 96 vs 83.
+// vs 32.4, FP16 38.0 vs 44.5.  D2Q9, us per step of a periodic box, one vs two:
+// FP32 1024^2 9.8 vs 8.1, 512^2 3.9 vs 3.5, FP16 1024^2 9.7 vs 7.0, 512^2 3.9 vs 3.0,
+// 256^2 2.45 vs 2.30.
 inline int vec_default(int lattice, int precision)
 {
-    if (lattice == 0 /* D2Q9 */ || precision == PREC_FP64) return 1;
-    if (precision == PREC_FP32) return lattice == 2 /* D3Q27 */ ? 2 : 1;
+    if (precision == PREC_FP64) return 1;
+    if (precision == PREC_FP32) return lattice == 1 /* D3Q19 */ ? 1 : 2;
     return 2;
 }
 // Default threads per block.  The vectorised kernel's blocks lie along x

@@ -1097,12 +1097,24 @@ static bool staging_wanted(const lbm_ctx *h)
     return h->staging == 1;
 }
 
-// Whether the vectorised kernel can update a grid: no cell-type mask, the
-// rrBGK collision, the default storage shift, and sponge layers (if any)
-// relaxing to the rest state through face layers only (its closed form)
-static bool vec_eligible(const StepParams &p)
+// Whether the vectorised kernel can update a grid with vec cells per thread: no
+// cell-type mask, the rrBGK collision of order 3, the default storage shift (or
+// a combination it takes one in), and sponge layers (if any) relaxing to the
+// rest state through face layers only (its closed form)
+static bool vec_eligible(const lbm_ctx *h, const StepParams &p, int vec)
 {
-    return !p.solid && !p.bgk && !p.shifted && (!p.any_sponge || (p.sponge_rest && !p.radial_on));
+    return !p.solid && !p.bgk && !p.order4 && (!p.shifted || vec_shift_supported(h->q, h->elem, vec)) &&
+           (!p.any_sponge || (p.sponge_rest && !p.radial_on));
+}
+
+// Cells per thread of the register kernels for a grid: the chosen (or default)
+// number where the vectorised kernel can run it, else 1 (the general kernel)
+static int pick_vec(const lbm_ctx *h, const StepParams &p)
+{
+    const int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
+    // (the vector path addresses a lattice with 32-bit offsets)
+    const bool off32 = (int64_t)h->q * p.ncell * (int64_t)h->elem < ((int64_t)1 << 31);
+    return vec > 1 && p.n[0] % vec == 0 && off32 && vec_available(h, vec) && vec_eligible(h, p, vec) ? vec : 1;
 }
 
 // Launch one update of a grid: the row-staged kernel where it is wanted and
@@ -1135,8 +1147,7 @@ static cudaError_t launch_update(lbm_ctx *h, const StepParams &p, const void *fi
             return e;
         }
     }
-    int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
-    if (!vec_eligible(p) || vec == 1 || !vec_available(h, vec) || p.n[0] % vec != 0) vec = 1;
+    const int vec = pick_vec(h, p);
     const int block = h->block > 0 ? h->block : block_default(vec, p.n[0]);
     h->launches += 1;
     if (vec == 1) return step_general(h, p, fin, fout, block);
@@ -1303,8 +1314,7 @@ static int refresh_after_set(lbm_ctx *h, int k)
 static cudaError_t aa_step(lbm_ctx *h, const StepParams &p)
 {
     const bool loc = h->aa_odd != 0;
-    int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
-    if (!vec_eligible(p) || vec == 1 || !vec_available(h, vec) || p.n[0] % vec != 0) vec = 1;
+    const int vec = pick_vec(h, p);
     const int block = h->block > 0 ? h->block : block_default(vec, p.n[0]);
     h->launches += 1;
     h->aa_odd ^= 1;
@@ -1762,8 +1772,15 @@ extern "C" int lbm_set_launch(lbm_handle h, int block, int cells_per_thread)
 extern "C" int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread)
 {
     CHECK_HANDLE(h);
-    int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
-    if (h->solid_d || vec == 1 || !vec_available(h, vec) || h->n[0] % vec != 0) vec = 1;
+    int vec = h->vec;
+    if (vec == 0) {  // the default: what level 0 runs as configured now
+        StepParams p;
+        const int rc = build_params(h, p);
+        if (rc != LBM_OK) return rc;
+        vec = pick_vec(h, p);
+    } else if (h->solid_d || !vec_available(h, vec) || h->n[0] % vec != 0) {
+        vec = 1;
+    }
     if (block) *block = h->block > 0 ? h->block : block_default(vec, h->n[0]);  // level 0
     if (cells_per_thread) *cells_per_thread = vec;
     return LBM_OK;

@@ -25,6 +25,7 @@
 
 #include <type_traits>
 
+#include "dispatch.h"
 #include "step.cuh"
 
 namespace rr {
@@ -249,8 +250,7 @@ struct GroupSt<__nv_bfloat16, 4> {
 };
 
 // ---------------------------------------------------------------------------
-// Rows whose y / z neighbour rows do not wrap around and that are not on a
-// non-periodic y / z face (1 <= y <= ny - 2, 1 <= z <= nz - 2): every
+// Rows of the vector path (vec_row): every
 // population is pulled from a fixed offset of the thread's own cell -- the
 // row x - xi_i in direction i's array, i times the direction stride
 // (p.st_off[1] bytes) from the lattice: one V-wide aligned load per
@@ -308,7 +308,7 @@ __device__ __forceinline__ RowOff row_offsets(const StepParams &p, int y, int z)
 {
     const int nx = p.n[0], ny = p.n[1], nz = p.n[2], nxy = nx * ny;
     RowOff o;
-    if (WR) {
+    if (WR || L::D == 2) {
         o.ym = y == 0 ? (ny - 1) * nx : -nx;
         o.yp = y == ny - 1 ? -(ny - 1) * nx : nx;
         o.zm = L::D == 2 ? 0 : (z == 0 ? (nz - 1) * nxy : -nxy);
@@ -392,8 +392,8 @@ __device__ __forceinline__ bool vec_load(const StepParams &p, const char *in0, i
         // its neighbour's populations), and the addresses stay inside the
         // lattice's allocation -- direction i >= 1 with xi_x > 0 reads at
         // index i ncell + src - 1 >= 0, and the last direction with xi_x < 0
-        // (D2Q9 7, D3Q19 16, D3Q27 26) pulls from a row before the last one,
-        // so i ncell + src + V < Q ncell.  A uniform branch, so no warp
+        // is not the last one (D2Q9 7, D3Q19 16) or pulls from a row before the
+        // last one (D3Q27 26), so i ncell + src + V < Q ncell.  A uniform branch, so no warp
         // diverges on it.
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) {
@@ -467,6 +467,17 @@ __device__ __forceinline__ void vec_store(const StepParams &p, char *bout, int x
     }
 }
 
+// Storage shift (lbm_set_storage_shift): dsh added to loaded populations (sign
+// 1), subtracted from those to be stored (-1); SH = false compiles to nothing
+template <class L, class C, bool SH>
+__device__ __forceinline__ void add_shift(const StepParams &p, C *g, C sign)
+{
+    if constexpr (SH) {
+#pragma unroll
+        for (int i = 0; i < L::Q; ++i) g[i] += sign * dsh<C>(p, i);
+    }
+}
+
 // Collide the V cells of a loaded vector and store them, one cell at a time
 // (gather, moments, coefficients, rebuild).  all_bulk: every cell of the
 // vector is bulk (no sponge, no boundary role), decided by the caller for a
@@ -475,7 +486,7 @@ __device__ __forceinline__ void vec_store(const StepParams &p, char *bout, int x
 // closed-form coefficients of a rest-state reference.  A node on a
 // non-periodic x face collides its neighbour's streamed populations: as they
 // are (outflow face) or with the face's density / velocity substituted.
-template <class L, class S, class C, int V, int G, int SP, int WR>
+template <class L, class S, class C, int V, int G, int SP, int WR, bool SH>
 __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out0, int x0, int y, int z,
                                                   const RowOff &ro, const VecIn<L, S, C, V> &r, bool all_bulk)
 {
@@ -499,6 +510,7 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
             Coef<C> cf;  // (unused in FP64, whose collision has a form of its own)
             if (all_bulk) {
                 gather_vec<L, S, C, V, SP>(r, k, g);
+                add_shift<L, C, SH>(p, g, C(1));
                 m = moments_pairs<L, C>(g);
                 if constexpr (!has_fp64_form<L, C>()) cf = coef_interior<L, C, false>(m, om, C(0));
             } else {
@@ -509,6 +521,7 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
                     gather_vec<L, S, C, V, SP>(r, k == 0 ? 1 : V - 2, g);
                 else
                     gather_vec<L, S, C, V, SP>(r, k, g);
+                add_shift<L, C, SH>(p, g, C(1));
                 m = moments_pairs<L, C>(g);
                 const int x = x0 + k;
                 const int inlet = !face ? -1 : (k == 0 ? (p.kind[0] != BC_OUTFLOW ? 0 : -1)
@@ -532,23 +545,40 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
             } else {
                 rebuild_all<L, C, false, !WR>(cf, o[kk]);
             }
+            add_shift<L, C, SH>(p, o[kk], C(-1));
         }
         vec_store<L, S, C, V, G, SP>(p, bout, x0, k0, ro, o);
     }
 }
 
-// Whether the vector path applies to row (y, z): its y / z neighbour rows do
-// not wrap and it is not on a non-periodic y / z face; for the AA steps its
-// neighbours are not face rows either.  The handle's sponge layers relax to
-// the rest state (the vector path's closed form) -- launch_update checks it.
+// Whether the vector path applies to row (y, z), and the row sy whose streamed
+// populations it collides.  3D: rows whose y / z neighbour rows do not wrap and
+// that are not on a non-periodic y / z face (for the AA steps, nor next to
+// one).  2D: the rows of a periodic y axis, wrapped around, and for the pull
+// also outflow face rows, which take the inward neighbour row's populations
+// as they are.  The other rows run the general update, V cells one after the
+// other.  (In 2D that took 1.0 us of a 1024 x 1024 FP16 step, 7.96 -> 6.95 us:
+// two rows, but they finish last; the 3D kernels lost 2 % at 384 x 256 x 256 to
+// the offsets that these rows need.)  The handle's sponge layers
+// relax to the rest state (the vector path's closed form) -- launch_update
+// checks it.
 template <class L, int SP>
-__device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z)
+__device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z, int &sy)
 {
     const int ny = p.n[1], nz = p.n[2];
-    bool ok = p.off32 && !p.order4 && y > 0 && y < ny - 1 && (L::D == 2 || (z > 0 && z < nz - 1));
+    sy = y;
+    bool ok = p.off32 && !p.order4;
+    if constexpr (L::D == 2) {
+        if (p.periodic[1]) return ok;
+        if (SP != kPull) return ok && y > 1 && y < ny - 2;
+        if (y == 0) { sy = 1; ok = ok && p.kind[2] == BC_OUTFLOW; }
+        if (y == ny - 1) { sy = y - 1; ok = ok && p.kind[3] == BC_OUTFLOW; }
+        return ok;
+    }
+    ok = ok && y > 0 && y < ny - 1 && z > 0 && z < nz - 1;
     if (SP != kPull) {
         if (!p.periodic[1]) ok = ok && y > 1 && y < ny - 2;
-        if (L::D == 3 && !p.periodic[2]) ok = ok && z > 1 && z < nz - 2;
+        if (!p.periodic[2]) ok = ok && z > 1 && z < nz - 2;
     }
     return ok;
 }
@@ -575,19 +605,20 @@ __device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z)
 // takes the vector path, the first and last rows' neighbours wrapped
 // (row_offsets), and no general update is compiled in.
 // ---------------------------------------------------------------------------
-template <class L, class S, class C, int V, int G, int SP = kPull, int WR = 0>
+template <class L, class S, class C, int V, int G, int SP = kPull, int WR = 0, bool SH = false>
 __device__ __forceinline__ void update_vec(const StepParams &p, const char *const *in, char *const *out, int x0,
                                            int y, int z)
 {
     const int nx = p.n[0];
     if (x0 >= nx) return;  // lanes past the row end
-    if (WR || vec_row<L, SP>(p, y, z)) {
-        const RowOff ro = row_offsets<L, WR>(p, y, z);
+    int sy = y;
+    if (WR || vec_row<L, SP>(p, y, z, sy)) {
+        const RowOff ro = row_offsets<L, WR>(p, sy, z);
         VecIn<L, S, C, V> r;
-        if (!vec_load<L, S, C, V, SP>(p, in[0], x0, y, z, ro, r)) return;
+        if (!vec_load<L, S, C, V, SP>(p, in[0], x0, sy, z, ro, r)) return;
         const bool bulk = y >= p.blo[1] && y < p.bhi[1] && z >= p.blo[2] && z < p.bhi[2] && x0 >= p.blo[0] &&
                           x0 + V <= p.bhi[0];
-        vec_collide_store<L, S, C, V, G, SP, WR>(p, out[0], x0, y, z, ro, r, bulk);
+        vec_collide_store<L, S, C, V, G, SP, WR, SH>(p, out[0], x0, y, z, ro, r, bulk);
         return;
     }
     if constexpr (!WR) {
@@ -623,10 +654,10 @@ struct VecGroup {
 // per thread.  Requires: no cell-type mask, nx % V == 0.
 // ---------------------------------------------------------------------------
 // Grid (x blocks of a row, ny, nz)
-template <class L, class S, class C, int V, int SP>
+template <class L, class S, class C, int V, int SP, bool SH = false>
 __global__ void __launch_bounds__(256, (VecMinBlocks<L, S, V, SP>::value)) k_stream_collide_vec(const __grid_constant__ StepParams p)
 {
-    update_vec<L, S, C, V, VecGroup<S, V>::value, SP>(p, p.in, p.out, (blockIdx.x * blockDim.x + threadIdx.x) * V,
+    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, 0, SH>(p, p.in, p.out, (blockIdx.x * blockDim.x + threadIdx.x) * V,
                                                       blockIdx.y, blockIdx.z);
 }
 
@@ -641,6 +672,12 @@ cudaError_t launch_stream_collide_vec(const StepParams &p, const void *fin, void
     dim3 g((p.n[0] / V + b - 1) / b, p.n[1], p.n[2]);
     StepParams q = p;
     set_bases<L, S>(q, fin, fout);
+    if constexpr (vec_shift_supported(L::Q, sizeof(S), V)) {
+        if (p.shifted && sp == kPull) {
+            k_stream_collide_vec<L, S, C, V, kPull, true><<<g, bd, 0, st>>>(q);
+            return cudaGetLastError();
+        }
+    }
     if (sp == kAAPush)
         k_stream_collide_vec<L, S, C, V, kAAPush><<<g, bd, 0, st>>>(q);
     else if (sp == kAALocal)

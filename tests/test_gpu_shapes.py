@@ -141,3 +141,56 @@ def test_fp64_collision_form(lattice, n, kinds, rho_ref):
     f = P.run(f, 3)
     got, _ = populations(c, "fp64")
     assert np.abs(got - f).max() < 1e-13
+
+
+@pytest.mark.parametrize("nx", [4, 6, 34, 62, 66, 130])
+@pytest.mark.parametrize("faces", ["periodic", "open x", "outflow y", "free-slip y"])
+@pytest.mark.parametrize("shift", [False, True])
+@pytest.mark.parametrize("lattice,prec", [(D2Q9, "fp32"), (D2Q9, "fp16"), (D2Q9, "bf16"), (D3Q19, "fp16"),
+                                          (D3Q27, "bf16")])
+def test_vector_rows_and_shift_against_the_general_kernel(lattice, prec, shift, faces, nx):
+    """The rows the 2D vector path takes (wrapped, outflow faces), the ones it
+    leaves, and the storage shift in the vector kernel: default shape against
+    one cell per thread.  FP32: 1e-5 of the largest deviation from the mean;
+    16-bit storage: one rounding of each stored value per step and the start
+    (2^-10, 2^-7 of the largest)."""
+    from paper_1710_02065_gb300 import lbm
+    n = (nx, 7, 1) if lattice == D2Q9 else (nx, 6, 5)
+    c = with_random_state(Case("rows", lattice, n, 0.6), seed=9, spread=0.05)
+    if faces == "open x":
+        c.faces = {0: (VELOCITY, (0.03, 0.0, 0.0), None), 1: (OUTFLOW, (0, 0, 0), None)}
+        c.sponges = {1: (2, 0.4)}
+    elif faces != "periodic":
+        kind = OUTFLOW if faces == "outflow y" else FREESLIP
+        c.faces = {2: (OUTFLOW, (0, 0, 0), None), 3: (kind, (0, 0, 0), None)}
+        c.sponges = {2: (3, 0.3)}
+    out = []
+    for shape in ((128, 1), None):
+        s = to_gpu(c, PRECS[prec])
+        if shift:
+            lbm.lbm_set_storage_shift(s.h, (0.05, 0.02, 0.0))
+        if shape:
+            lbm.lbm_set_launch(s.h, *shape)
+        assert lbm.lbm_get_launch(s.h)[1] == (1 if shape else 2)
+        s.step(3)
+        lbm.lbm_sync(s.h)
+        out.append(s.populations())
+        s.close()
+    dev = np.abs(out[0] - out[0].mean(axis=1, keepdims=True)).max()
+    tol = {"fp32": 1e-5, "fp16": 4 * 2.0 ** -10, "bf16": 4 * 2.0 ** -7}[prec]
+    assert np.abs(out[1] - out[0]).max() <= tol * dev
+
+
+@pytest.mark.parametrize("option", ["order 4", "sponge reference", "solid", "odd row"])
+def test_options_the_vector_kernel_leaves_run_the_general_one(option):
+    from paper_1710_02065_gb300 import lbm
+    c = open_box(D2Q9, (33 if option == "odd row" else 34, 7, 1))
+    if option == "sponge reference":
+        c.u_ref = (0.03, 0.0, 0.0)
+    if option == "solid":
+        c.solid = np.eye(1, c.ncell, 50, dtype=np.uint8)[0]
+    s = to_gpu(c, PRECS["fp32"])
+    if option == "order 4":
+        lbm.lbm_set_hermite_order(s.h, 4)
+    assert lbm.lbm_get_launch(s.h) == (128, 1)
+    s.close()
