@@ -48,7 +48,7 @@ struct lbm_ctx {
     int level_overlap = 1;
     cudaStream_t side = nullptr;
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
-    int sms = 0;  // SMs of the device (set with the second stream)
+    int sms = 0;  // SMs of the device
     void *f[2] = {nullptr, nullptr};
     int cur = 0;
     uint8_t *solid_d = nullptr;
@@ -540,6 +540,13 @@ extern "C" int lbm_create(lbm_handle *out, int lattice, const int extents[3], do
         cudaGetLastError();
         release(h);
         return fail(nullptr, LBM_ENOMEM, "allocating the sponge tables failed");
+    }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        release(h);
+        return fail(nullptr, LBM_ECUDA, "reading the device's SM count failed");
     }
     // rest state: rho = 1, u = 0 is g = f - w = 0 in every storage format
     for (int k = 0; k < 2; ++k)
@@ -1367,9 +1374,6 @@ static cudaError_t ensure_side_stream(lbm_ctx *h)
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, greatest);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->join_ev, cudaEventDisableTiming);
-    int dev = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
     return e;
 }
 
@@ -1516,6 +1520,13 @@ extern "C" int lbm_step(lbm_handle h, int64_t n)
     int rc = build_params(h, params[0]);
     if (rc != LBM_OK) return rc;
     for (int k = 1; k < nlevels(h); ++k) fine_params(h, k, params[(size_t)k]);
+    // The updates of a single level follow one another in the stream: chained
+    // launches (with refined levels an update waits for two streams; a caller's
+    // own capture gets plain launches)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusActive;
+    if (h->stream && h->levels.empty()) CUDA_TRY(h, cudaStreamIsCapturing(h->stream, &capturing));
+    params[0].chained = capturing == cudaStreamCaptureStatusNone ? 1 : 0;
+    params[0].chain_sms = h->sms;
     // Without inlet noise every step of a pair has the same parameters, so
     // pairs of steps are replayed from captured graphs (needs a stream other
     // than the legacy default one).  Every refined level returns to the same

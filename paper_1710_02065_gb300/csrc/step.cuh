@@ -102,7 +102,47 @@ struct StepParams {
     int shifted;
     float dsh_f[kMaxQ];
     double dsh_d[kMaxQ];
+    // chained launch (launch_step): 0 no; 1 yes; 2 yes, and the next launch may
+    // become resident as soon as this one is (set by launch_step).  chain_sms:
+    // SMs of the device
+    int chained, chain_sms;
 };
+
+// The pull updates of a single level are chained launches: the next one is
+// launched while the one before it still runs and begins by waiting until that
+// one has ended and its writes are visible.  Nothing is read or written before
+// the wait, and every launch of a chain waits, so each runs after all before
+// it, as unchained launches do; what is hidden is the launch itself.
+__device__ __forceinline__ void chain_begin(const StepParams &p)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.chained > 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch `plain`, or as a chained launch its twin `chain`.  The next launch
+// starts when the blocks of this one have ended, or (chained = 2) as soon as all
+// of them are resident: where two launches fit on the device together
+// (at most 512 threads per SM each), its blocks then wait on their SMs.  With
+// more blocks than that the early start can be a loss.  GB300, us per step, unchained / chained (1 / 2): D2Q9
+// FP64 128^2 pulse 5.06 / 4.83 / 4.67, FP16 1024^2 pulse 8.1 / 8.0 / 9.3; the jets,
+// whose steps are launched one by one (1 only): D3Q27 FP16 192 x 128 x 128 79.2 /
+// 78.1, D3Q19 FP64 96 x 64 x 64 144.4 / 141.8.
+template <class K>
+inline cudaError_t launch_step(K plain, K chain, dim3 grid, dim3 block, cudaStream_t st, StepParams p)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = p.chained ? 1 : 0;
+    if (p.chained && (int64_t)grid.x * grid.y * grid.z * block.x <= 512 * (int64_t)p.chain_sms) p.chained = 2;
+    cudaLaunchKernelEx(&c, p.chained ? chain : plain, p);
+    return cudaGetLastError();
+}
 
 template <class C>
 __device__ __forceinline__ C dsh(const StepParams &p, int i);
@@ -498,7 +538,7 @@ __device__ __forceinline__ void cell_collide(const StepParams &p, const Mom<C> &
         if (BGK) o[i] = fmac(keep, g[i], o[i]);
 }
 
-template <class L, class S, class C, bool BGK = false, int MASK = kMaskLinks>
+template <class L, class S, class C, bool BGK = false, int MASK = kMaskLinks, bool CH = false>
 __device__ __forceinline__ void update_cell(const StepParams &p, const char *const *in, char *const *out,
                                             int x, int y, int z)
 {
@@ -565,7 +605,7 @@ __device__ __forceinline__ void update_cell(const StepParams &p, const char *con
             const unsigned src = X + nx * Y + nxy * Z;
             // a bounced population is stored in the opposite direction's array (and shift)
             const int k = (i != 0 && (solid[src] & MASK_TYPE) == MASK_SOLID) ? opp<L>(i) : i;
-            g[i] = Store<S>::ld((const S *)in[k] + (k == i ? src : scell));
+            g[i] = Store<S>::template ld<CH>((const S *)in[k] + (k == i ? src : scell));
             if (p.shifted) g[i] += dsh<C>(p, k);
         }
     } else {
@@ -574,7 +614,7 @@ __device__ __forceinline__ void update_cell(const StepParams &p, const char *con
             const unsigned X = L::cx(i) > 0 ? xm : (L::cx(i) < 0 ? xp : sx);
             const unsigned Y = L::cy(i) > 0 ? ym : (L::cy(i) < 0 ? yp : sy);
             const unsigned Z = L::D == 2 ? 0u : (L::cz(i) > 0 ? zm : (L::cz(i) < 0 ? zp : sz));
-            g[i] = Store<S>::ld((const S *)in[i] + (X + nx * Y + nxy * Z));
+            g[i] = Store<S>::template ld<CH>((const S *)in[i] + (X + nx * Y + nxy * Z));
         }
         if (p.shifted) {
 #pragma unroll
@@ -810,25 +850,27 @@ cudaError_t launch_aa_unswap(const StepParams &p, void *f, cudaStream_t st)
 
 // General kernel: one thread per cell; MASK: cell-type handling (above);
 // BGK = true is the plain LBM-BGK collision (Eq. standardLB).
-template <class L, class S, class C, bool BGK, int MASK>
+template <class L, class S, class C, bool BGK, int MASK, bool CH = false>
 __global__ void __launch_bounds__(256) k_stream_collide(const __grid_constant__ StepParams p)
 {
+    if constexpr (CH) chain_begin(p);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.n[0]) return;
-    update_cell<L, S, C, BGK, MASK>(p, p.in, p.out, x, blockIdx.y, blockIdx.z);
+    update_cell<L, S, C, BGK, MASK, CH>(p, p.in, p.out, x, blockIdx.y, blockIdx.z);
 }
 
 // The same update with one thread per cell of the whole lattice, for rows
 // whose length would leave many threads of their blocks idle (a 129-cell row
 // in 128-thread blocks idles half of them); rrBGK only.
-template <class L, class S, class C, int MASK>
+template <class L, class S, class C, int MASK, bool CH = false>
 __global__ void __launch_bounds__(256) k_stream_collide_lin(const __grid_constant__ StepParams p)
 {
+    if constexpr (CH) chain_begin(p);
     const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (unsigned)p.ncell) return;
     const unsigned nx = p.n[0], nxy = nx * (unsigned)p.n[1];
     const unsigned z = t / nxy, r = t - z * nxy, y = r / nx;
-    update_cell<L, S, C, false, MASK>(p, p.in, p.out, (int)(r - y * nx), (int)y, (int)z);
+    update_cell<L, S, C, false, MASK, CH>(p, p.in, p.out, (int)(r - y * nx), (int)y, (int)z);
 }
 
 // Launch wrapper: one thread per cell, blocks along x; p.bgk selects the
@@ -852,7 +894,7 @@ cudaError_t launch_stream_collide(const StepParams &p, const void *fin, void *fo
         else if (mode == kMaskSkip)
             k_stream_collide_lin<L, S, C, kMaskSkip><<<gl, b, 0, st>>>(q);
         else
-            k_stream_collide_lin<L, S, C, kMaskNone><<<gl, b, 0, st>>>(q);
+            return launch_step(k_stream_collide_lin<L, S, C, kMaskNone>, k_stream_collide_lin<L, S, C, kMaskNone, true>, gl, b, st, q);
         return cudaGetLastError();
     }
     if (p.bgk) {
@@ -866,7 +908,8 @@ cudaError_t launch_stream_collide(const StepParams &p, const void *fin, void *fo
         else if (mode == kMaskSkip)
             k_stream_collide<L, S, C, false, kMaskSkip><<<g, b, 0, st>>>(q);
         else
-            k_stream_collide<L, S, C, false, kMaskNone><<<g, b, 0, st>>>(q);
+            return launch_step(k_stream_collide<L, S, C, false, kMaskNone>, k_stream_collide<L, S, C, false, kMaskNone, true>, g, b, st,
+                               q);
     }
     return cudaGetLastError();
 }

@@ -154,19 +154,22 @@ struct Raw;
 template <>
 struct Raw<double, 2> {
     using T = double2;
-    __device__ static T ld(const double *p) { return __ldg(reinterpret_cast<const double2 *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const double *p) { return ld_pop<CH>(reinterpret_cast<const double2 *>(p)); }
     __device__ static double get(const T &v, int k) { return k == 0 ? v.x : v.y; }
 };
 template <>
 struct Raw<float, 2> {
     using T = float2;
-    __device__ static T ld(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const float *p) { return ld_pop<CH>(reinterpret_cast<const float2 *>(p)); }
     __device__ static float get(const T &v, int k) { return k == 0 ? v.x : v.y; }
 };
 template <>
 struct Raw<float, 4> {
     using T = float4;
-    __device__ static T ld(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const float *p) { return ld_pop<CH>(reinterpret_cast<const float4 *>(p)); }
     __device__ static float get(const T &v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w)); }
 };
 __device__ __forceinline__ float half_lo(unsigned w) { return __low2float(*reinterpret_cast<const __half2 *>(&w)); }
@@ -174,13 +177,15 @@ __device__ __forceinline__ float half_hi(unsigned w) { return __high2float(*rein
 template <>
 struct Raw<__half, 2> {
     using T = unsigned;
-    __device__ static T ld(const __half *p) { return __ldg(reinterpret_cast<const unsigned *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const __half *p) { return ld_pop<CH>(reinterpret_cast<const unsigned *>(p)); }
     __device__ static float get(const T &v, int k) { return k == 0 ? half_lo(v) : half_hi(v); }
 };
 template <>
 struct Raw<__half, 4> {
     using T = uint2;
-    __device__ static T ld(const __half *p) { return __ldg(reinterpret_cast<const uint2 *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const __half *p) { return ld_pop<CH>(reinterpret_cast<const uint2 *>(p)); }
     __device__ static float get(const T &v, int k)
     {
         return k == 0 ? half_lo(v.x) : (k == 1 ? half_hi(v.x) : (k == 2 ? half_lo(v.y) : half_hi(v.y)));
@@ -191,13 +196,15 @@ __device__ __forceinline__ float bf_hi(unsigned w) { return __uint_as_float(w & 
 template <>
 struct Raw<__nv_bfloat16, 2> {
     using T = unsigned;
-    __device__ static T ld(const __nv_bfloat16 *p) { return __ldg(reinterpret_cast<const unsigned *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const __nv_bfloat16 *p) { return ld_pop<CH>(reinterpret_cast<const unsigned *>(p)); }
     __device__ static float get(const T &v, int k) { return k == 0 ? bf_lo(v) : bf_hi(v); }
 };
 template <>
 struct Raw<__nv_bfloat16, 4> {
     using T = uint2;
-    __device__ static T ld(const __nv_bfloat16 *p) { return __ldg(reinterpret_cast<const uint2 *>(p)); }
+    template <bool CH = false>
+    __device__ static T ld(const __nv_bfloat16 *p) { return ld_pop<CH>(reinterpret_cast<const uint2 *>(p)); }
     __device__ static float get(const T &v, int k)
     {
         return k == 0 ? bf_lo(v.x) : (k == 1 ? bf_hi(v.x) : (k == 2 ? bf_lo(v.y) : bf_hi(v.y)));
@@ -348,7 +355,7 @@ __device__ __forceinline__ const S *vec_row_ptr(const char *bin, int i, const Ro
 
 // Loads of one thread's vector (x0, y, z) of such a row; false when a
 // checked build finds an index outside the lattice (nothing loaded).
-template <class L, class S, class C, int V, int SP>
+template <class L, class S, class C, int V, int SP, bool CH>
 __device__ __forceinline__ bool vec_load(const StepParams &p, const char *in0, int x0, int y, int z,
                                          const RowOff &ro, VecIn<L, S, C, V> &r)
 {
@@ -385,7 +392,7 @@ __device__ __forceinline__ bool vec_load(const StepParams &p, const char *in0, i
     if (SP == kAALocal) {
 #pragma unroll
         for (int i = 0; i < L::Q; ++i)
-            r.v[i] = RW::ld(reinterpret_cast<const S *>(bin + (size_t)opp<L>(i) * dstride));
+            r.v[i] = RW::template ld<CH>(reinterpret_cast<const S *>(bin + (size_t)opp<L>(i) * dstride));
     } else if (!p.periodic[0]) {
         // The edge values at x0 - 1 / x0 + V are read unconditionally: on the
         // x faces (x0 = 0, x0 + V = nx) they are not used (the face node takes
@@ -398,17 +405,17 @@ __device__ __forceinline__ bool vec_load(const StepParams &p, const char *in0, i
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) {
             const S *row = vec_row_ptr<L, S, SP>(bin, i, ro, dstride);
-            r.v[i] = RW::ld(row);
-            if (L::cx(i) > 0) r.e[i] = Store<S>::ld(row - 1);
-            if (L::cx(i) < 0) r.e[i] = Store<S>::ld(row + V);
+            r.v[i] = RW::template ld<CH>(row);
+            if (L::cx(i) > 0) r.e[i] = Store<S>::template ld<CH>(row - 1);
+            if (L::cx(i) < 0) r.e[i] = Store<S>::template ld<CH>(row + V);
         }
     } else {
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) {
             const S *row = vec_row_ptr<L, S, SP>(bin, i, ro, dstride);
-            r.v[i] = RW::ld(row);
-            if (L::cx(i) > 0) r.e[i] = Store<S>::ld(row + dl);
-            if (L::cx(i) < 0) r.e[i] = Store<S>::ld(row + dr);
+            r.v[i] = RW::template ld<CH>(row);
+            if (L::cx(i) > 0) r.e[i] = Store<S>::template ld<CH>(row + dl);
+            if (L::cx(i) < 0) r.e[i] = Store<S>::template ld<CH>(row + dr);
         }
     }
     return true;
@@ -605,7 +612,7 @@ __device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z, int &
 // takes the vector path, the first and last rows' neighbours wrapped
 // (row_offsets), and no general update is compiled in.
 // ---------------------------------------------------------------------------
-template <class L, class S, class C, int V, int G, int SP = kPull, int WR = 0, bool SH = false>
+template <class L, class S, class C, int V, int G, int SP = kPull, int WR = 0, bool SH = false, bool CH = false>
 __device__ __forceinline__ void update_vec(const StepParams &p, const char *const *in, char *const *out, int x0,
                                            int y, int z)
 {
@@ -615,7 +622,7 @@ __device__ __forceinline__ void update_vec(const StepParams &p, const char *cons
     if (WR || vec_row<L, SP>(p, y, z, sy)) {
         const RowOff ro = row_offsets<L, WR>(p, sy, z);
         VecIn<L, S, C, V> r;
-        if (!vec_load<L, S, C, V, SP>(p, in[0], x0, sy, z, ro, r)) return;
+        if (!vec_load<L, S, C, V, SP, CH>(p, in[0], x0, sy, z, ro, r)) return;
         const bool bulk = y >= p.blo[1] && y < p.bhi[1] && z >= p.blo[2] && z < p.bhi[2] && x0 >= p.blo[0] &&
                           x0 + V <= p.bhi[0];
         vec_collide_store<L, S, C, V, G, SP, WR, SH>(p, out[0], x0, y, z, ro, r, bulk);
@@ -625,7 +632,7 @@ __device__ __forceinline__ void update_vec(const StepParams &p, const char *cons
 #pragma unroll 1
         for (int k = 0; k < V; ++k) {
             if (SP == kPull)
-                update_cell<L, S, C, false, kMaskNone>(p, in, out, x0 + k, y, z);
+                update_cell<L, S, C, false, kMaskNone, CH>(p, in, out, x0 + k, y, z);
             else
                 update_cell_aa<L, S, C, false, kMaskNone, SP == kAALocal>(p, out, x0 + k, y, z);
         }
@@ -654,11 +661,13 @@ struct VecGroup {
 // per thread.  Requires: no cell-type mask, nx % V == 0.
 // ---------------------------------------------------------------------------
 // Grid (x blocks of a row, ny, nz)
-template <class L, class S, class C, int V, int SP, bool SH = false>
+template <class L, class S, class C, int V, int SP, bool SH = false, bool CH = false>
 __global__ void __launch_bounds__(256, (VecMinBlocks<L, S, V, SP>::value)) k_stream_collide_vec(const __grid_constant__ StepParams p)
 {
-    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, 0, SH>(p, p.in, p.out, (blockIdx.x * blockDim.x + threadIdx.x) * V,
-                                                      blockIdx.y, blockIdx.z);
+    if constexpr (CH) chain_begin(p);
+    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, 0, SH, CH>(p, p.in, p.out,
+                                                                 (blockIdx.x * blockDim.x + threadIdx.x) * V,
+                                                                 blockIdx.y, blockIdx.z);
 }
 
 // sp: kPull (fin read, fout written) or an AA step type (fin == fout)
@@ -673,17 +682,17 @@ cudaError_t launch_stream_collide_vec(const StepParams &p, const void *fin, void
     StepParams q = p;
     set_bases<L, S>(q, fin, fout);
     if constexpr (vec_shift_supported(L::Q, sizeof(S), V)) {
-        if (p.shifted && sp == kPull) {
-            k_stream_collide_vec<L, S, C, V, kPull, true><<<g, bd, 0, st>>>(q);
-            return cudaGetLastError();
-        }
+        if (p.shifted && sp == kPull)
+            return launch_step(k_stream_collide_vec<L, S, C, V, kPull, true>,
+                               k_stream_collide_vec<L, S, C, V, kPull, true, true>, g, bd, st, q);
     }
+    if (sp == kPull)
+        return launch_step(k_stream_collide_vec<L, S, C, V, kPull>, k_stream_collide_vec<L, S, C, V, kPull, false, true>, g,
+                           bd, st, q);
     if (sp == kAAPush)
         k_stream_collide_vec<L, S, C, V, kAAPush><<<g, bd, 0, st>>>(q);
-    else if (sp == kAALocal)
-        k_stream_collide_vec<L, S, C, V, kAALocal><<<g, bd, 0, st>>>(q);
     else
-        k_stream_collide_vec<L, S, C, V, kPull><<<g, bd, 0, st>>>(q);
+        k_stream_collide_vec<L, S, C, V, kAALocal><<<g, bd, 0, st>>>(q);
     return cudaGetLastError();
 }
 

@@ -194,3 +194,30 @@ def test_options_the_vector_kernel_leaves_run_the_general_one(option):
         lbm.lbm_set_hermite_order(s.h, 4)
     assert lbm.lbm_get_launch(s.h) == (128, 1)
     s.close()
+
+
+@pytest.mark.parametrize("noise", [0.0, 0.01])
+@pytest.mark.parametrize("lattice,prec,n", [(D2Q9, "fp64", (16, 16, 1)), (D2Q9, "fp16", (256, 250, 1)),
+                                            (D2Q9, "fp32", (512, 640, 1)), (D3Q19, "fp32", (33, 40, 39)),
+                                            (D3Q19, "bf16", (160, 64, 60)), (D3Q27, "fp16", (64, 48, 40))])
+def test_chained_launches_are_the_plain_ones_bit_for_bit(lattice, prec, n, noise):
+    """Steps on a stream of their own run as chained launches (captured pairs
+    without inlet noise, single launches with it; lattices below and above the
+    early-start size), on the legacy stream as plain ones."""
+    from paper_1710_02065_gb300 import lbm
+    c = open_box(lattice, n)
+    out = []
+    for stream in (0, torch.cuda.Stream().cuda_stream):
+        s = lbm.Solver(c.lattice, c.n, c.tau, PRECS[prec], stream=stream)
+        for face, spec in c.faces.items():
+            lbm.lbm_set_boundary(s.h, face, *spec)
+        for face, (w, chi) in c.sponges.items():
+            lbm.lbm_set_sponge(s.h, face, w, chi)
+        lbm.lbm_set_inlet_noise(s.h, 3, noise)
+        s.set_populations(c.f0)
+        s.step(67)
+        s.step(3)
+        lbm.lbm_sync(s.h)
+        out.append(s.populations())
+        s.close()
+    assert np.isfinite(out[0]).all() and np.array_equal(out[0], out[1])
