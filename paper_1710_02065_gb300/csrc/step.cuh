@@ -59,6 +59,7 @@ struct StepParams {
     double omega;  // 1 - 1/tau
     const uint8_t *solid;  // device, or null
     int any_solid;         // the mask holds solid cells (else only fixed ones)
+    int back;  // sweep the rows from the last to the first (sweep_y)
     int64_t step;
     // bulk box: cells with blo[a] <= c[a] < bhi[a] on every axis have no
     // boundary role and no sponge (filled by the host from faces and layers)
@@ -73,6 +74,10 @@ struct StepParams {
     double jet_ref[6];
     // D2Q9: include the optional fourth-order H_xxyy term (rrBGK only)
     int order4;
+    // chained launch (launch_step): 0 no; 1 yes; 2 yes, and the next launch may
+    // become resident as soon as this one is (set by launch_step).  (back and
+    // chained fill padding: the members behind stay where they were.)
+    int chained;
     // per-direction base addresses of the lattice read (in) and written (out):
     // in[i] = f_in + i * ncell elements, i < Q <= kMaxQ; filled by the launchers
     const char *in[kMaxQ];
@@ -102,11 +107,24 @@ struct StepParams {
     int shifted;
     float dsh_f[kMaxQ];
     double dsh_d[kMaxQ];
-    // chained launch (launch_step): 0 no; 1 yes; 2 yes, and the next launch may
-    // become resident as soon as this one is (set by launch_step).  chain_sms:
-    // SMs of the device
-    int chained, chain_sms;
+    int chain_sms;  // (host) SMs of the device
 };
+
+// Row and plane of a block, and (one thread per cell of the whole lattice) its
+// number.  Consecutive steps sweep the lattice in opposite directions: the rows
+// written last by one step are still in L2 when the next one starts with them.
+__device__ __forceinline__ int sweep_y(const StepParams &p)
+{
+    return p.back ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
+}
+__device__ __forceinline__ int sweep_z(const StepParams &p)
+{
+    return p.back ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;
+}
+__device__ __forceinline__ unsigned sweep_x(const StepParams &p)
+{
+    return p.back ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+}
 
 // The pull updates of a single level are chained launches: the next one is
 // launched while the one before it still runs and begins by waiting until that
@@ -772,7 +790,7 @@ __global__ void __launch_bounds__(256) k_stream_collide_aa(const __grid_constant
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.n[0]) return;
-    update_cell_aa<L, S, C, BGK, MASK, LOC>(p, p.out, x, blockIdx.y, blockIdx.z);
+    update_cell_aa<L, S, C, BGK, MASK, LOC>(p, p.out, x, sweep_y(p), sweep_z(p));
 }
 
 // Launch one AA step (loc: the local step, else gather-push) of the lattice f
@@ -856,7 +874,7 @@ __global__ void __launch_bounds__(256) k_stream_collide(const __grid_constant__ 
     if constexpr (CH) chain_begin(p);
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= p.n[0]) return;
-    update_cell<L, S, C, BGK, MASK, CH>(p, p.in, p.out, x, blockIdx.y, blockIdx.z);
+    update_cell<L, S, C, BGK, MASK, CH>(p, p.in, p.out, x, sweep_y(p), sweep_z(p));
 }
 
 // The same update with one thread per cell of the whole lattice, for rows
@@ -866,7 +884,7 @@ template <class L, class S, class C, int MASK, bool CH = false>
 __global__ void __launch_bounds__(256) k_stream_collide_lin(const __grid_constant__ StepParams p)
 {
     if constexpr (CH) chain_begin(p);
-    const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned t = sweep_x(p) * blockDim.x + threadIdx.x;
     if (t >= (unsigned)p.ncell) return;
     const unsigned nx = p.n[0], nxy = nx * (unsigned)p.n[1];
     const unsigned z = t / nxy, r = t - z * nxy, y = r / nx;

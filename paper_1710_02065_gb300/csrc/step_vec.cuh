@@ -665,9 +665,8 @@ template <class L, class S, class C, int V, int SP, bool SH = false, bool CH = f
 __global__ void __launch_bounds__(256, (VecMinBlocks<L, S, V, SP>::value)) k_stream_collide_vec(const __grid_constant__ StepParams p)
 {
     if constexpr (CH) chain_begin(p);
-    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, 0, SH, CH>(p, p.in, p.out,
-                                                                 (blockIdx.x * blockDim.x + threadIdx.x) * V,
-                                                                 blockIdx.y, blockIdx.z);
+    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, 0, SH, CH>(
+        p, p.in, p.out, (blockIdx.x * blockDim.x + threadIdx.x) * V, sweep_y(p), sweep_z(p));
 }
 
 // sp: kPull (fin read, fout written) or an AA step type (fin == fout)
