@@ -832,14 +832,16 @@ __device__ __forceinline__ Coef<C> coef_interior(const Mom<C> &m, C om, C chi, b
 //   - with T_ab = A3_abb / 4 = u_a A'_bb + 2 u_b q'_ab, k_a = j_a / 12 and
 //     X_ab = T_ab + k_a, an edge direction's odd part is X_ab + X_ba (or their
 //     difference) and a face direction's 2 (k_a - T_ab - T_ac);
-//   - 1 / rho is one third-order correction x (1 + e + e^2), e = 1 - rho x, of a
-//     single-precision reciprocal x (|e| < 2^-23, so the rest is below 2^-68).
+//   - 1 / rho is one step of Chebyshev's method, r (1 + e + e^2) with e = 1 - rho r,
+//     from a single-precision reciprocal r (recip_fma).
 // D3Q19: 155 FP64 operations per bulk cell (from 175); D2Q9: 72 (from 92).
 // (Adding k_a inside T_ab's multiply-adds would save six more, but a face
 // direction then subtracts it again: 1.5 times the rounding error.)
 // Every operation is written with its rounding, so every kernel gives the
-// same bits; against 80-bit arithmetic the error of u after 40 steps is the
-// same as before (2.0e-15).  With the routes of cell_collide, GB300: D3Q19 jet
+// same bits.  Error against extended precision over ten runs of 100 to 200 steps
+// (periodic boxes and inlet / outflow channels of both lattices), relative to that of
+// coef_interior + rebuild_all: density 0.93 to 1.09, velocity 0.86 to 1.03.
+// With the routes of cell_collide, GB300: D3Q19 jet
 // 96 x 64 x 64 172.8 -> 141 us per step, 192 x 128 x 128 1.17 -> 1.02 ms; D2Q9
 // 128 x 128 5.1 -> 5.0 us (launch and latency).
 // chi = 0 gives the bulk result bit for bit.
@@ -850,11 +852,24 @@ __host__ __device__ constexpr bool has_fp64_form()
     return sizeof(C) == 8 && L::Q <= 19;
 }
 
+// 1 / x for normal |x| < 2^1022: Chebyshev's third-order method for the root of
+// 1 / r - x, from a single-precision reciprocal of x scaled to [1, 2) (x itself may
+// lie outside the single-precision range).  |e| < 2^-22 (two roundings to 24
+// bits), so the rest e^3 is below 2^-66 of the result, next to its last rounding.
+// Infinity for 0 and subnormal x, 0 for the largest, infinities and NaN.  The
+// scaling is on the integer pipe.  GB300, us per pass without the scaling / with a
+// branch to the quotient beyond single precision / as here: D2Q9 128 x 128 pulse
+// 884 / 894 / 891, D3Q19 96 x 64 x 64 jet 14201 / 14306 / 13690.
 __device__ __forceinline__ double recip_fma(double x)
 {
-    const double r = (double)__frcp_rn((float)x);
-    const double e = __fma_rn(-x, r, 1.0);
-    return __fma_rn(r, __fma_rn(e, e, e), r);
+    const int hi = __double2hiint(x), ex = hi & 0x7ff00000, sign = hi & (int)0x80000000;
+    const double m = __hiloint2double((hi & (int)0x800fffff) | 0x3ff00000, __double2loint(x));
+    const double r = (double)__frcp_rn((float)m);
+    const double e = __fma_rn(-m, r, 1.0);
+    const double q = __fma_rn(r, __fma_rn(e, e, e), r);
+    const bool normal = (unsigned)ex - 0x00100000u <= 0x7fc00000u - 0x00100000u;  // exponents 1 to 2044
+    return __hiloint2double(normal ? __double2hiint(q) + (0x3ff00000 - ex) : sign | (ex ? 0 : 0x7ff00000),
+                            normal ? __double2loint(q) : 0);
 }
 
 template <class L, bool SPONGE>
