@@ -590,7 +590,8 @@ int lbm_load(lbm_handle h, const char *path);
  * populations).  lbm_server_submit queues it (the initial fields are copied).
  * Each lbm_server_run call is one round: queued requests are admitted in
  * arrival order, first fit, while their population lattices (two, or one
- * with the AA pattern) fit in the HBM budget and a slot is free; then every
+ * with the AA pattern) fit in the HBM budget and a slot is free (a request
+ * that finds device memory short stays queued for the next round); then every
  * active request advances by up to `steps` steps in one CUDA-graph replay of
  * batched updates (one persistent launch per (lattice, precision) group, plus
  * a per-request step counter), a request stopping exactly at its own step
@@ -610,6 +611,12 @@ int lbm_load(lbm_handle h, const char *path);
  *   lbm_server_set_streaming : LBM_STREAM_PULL (default) or LBM_STREAM_AA for
  *                       requests admitted from now on (one lattice each, so
  *                       the budget holds twice the cells)
+ *   lbm_server_set_host_memory : bounds of the page-locked host memory that
+ *                       holds requests' fields: submitted requests take it
+ *                       while at most lend_bytes are in use (default 1 GiB; a
+ *                       request beyond it waits in pageable memory), and at
+ *                       most keep_bytes (default 256 MiB) are kept for later
+ *                       requests
  *   lbm_server_set_launch : launch shape of the (lattice, precision) group's
  *                       batched update from the next round on: cells_per_lane
  *                       1 or 2 (0: 2; a request with an odd row length, or
@@ -651,6 +658,7 @@ const char *lbm_server_last_error(lbm_server_handle s);
 int lbm_server_submit(lbm_server_handle s, const lbm_request *req, int64_t *id);
 int lbm_server_run(lbm_server_handle s, int64_t steps, int *completed);
 int lbm_server_set_streaming(lbm_server_handle s, int pattern);
+int lbm_server_set_host_memory(lbm_server_handle s, size_t lend_bytes, size_t keep_bytes);
 int lbm_server_set_launch(lbm_server_handle s, int lattice, int precision, int cells_per_lane, int warps_per_block);
 int lbm_server_get_launch(lbm_server_handle s, int lattice, int precision, int *cells_per_lane, int *warps_per_block);
 int lbm_server_poll(lbm_server_handle s, int64_t id, int *state, int64_t *steps_done);

@@ -214,15 +214,15 @@ struct lbm_server {
     std::vector<std::pair<double *, size_t>> blocks;  // page-locked blocks kept for reuse
     std::map<double *, size_t> held;     // blocks in use by requests
     size_t kept = 0, held_bytes = 0;
+    size_t host_lend = size_t(1) << 30, host_keep = size_t(256) << 20;  // lbm_server_set_host_memory
     std::string err;
 };
 
 // Page-locked host blocks.  Allocating and freeing one per request cost more
 // than its copies: the blocks of finished requests are kept for the next ones,
-// at most kPinnedKept bytes of them, and given back when the server is
-// destroyed.  Queued requests hold at most kPinnedMax bytes of blocks.
-constexpr size_t kPinnedKept = size_t(256) << 20, kPinnedMax = size_t(1) << 30;
-
+// at most host_keep bytes of them, and given back when the server is
+// destroyed.  A submitted request takes one while requests hold at most
+// host_lend bytes of them.
 static size_t host_bytes(const Request *r) { return sizeof(double) * 4 * (size_t)r->ncell; }
 
 // A block of at least `bytes` (null: allocation failed)
@@ -256,7 +256,7 @@ static void return_block(lbm_server *s, double *b)
     const size_t size = it->second;
     s->held.erase(it);
     s->held_bytes -= size;
-    if (s->kept + size > kPinnedKept) {
+    if (s->kept + size > s->host_keep) {
         cudaFreeHost(b);
         return;
     }
@@ -422,7 +422,7 @@ extern "C" int lbm_server_submit(lbm_server_handle s, const lbm_request *req, in
         return sfail(s, LBM_EINVAL, "request needs %zu bytes, more than the whole budget (%zu)", need, s->budget);
     }
     const size_t N = (size_t)r->ncell;
-    if (s->held_bytes + host_bytes(r) <= kPinnedMax) r->host = take_block(s, host_bytes(r));
+    if (s->held_bytes + host_bytes(r) <= s->host_lend) r->host = take_block(s, host_bytes(r));
     if (!r->host) r->pageable.resize(4 * N);
     double *h = r->host ? r->host : r->pageable.data();
     if (req->rho)
@@ -440,10 +440,26 @@ extern "C" int lbm_server_submit(lbm_server_handle s, const lbm_request *req, in
     return LBM_OK;
 }
 
+// Initial populations of a request from its host fields (device memory short of
+// the staging buffer of pageable fields: cudaErrorMemoryAllocation)
+static cudaError_t init_request(lbm_server *s, Request *r)
+{
+    // the kernel reads a page-locked block over the host link
+    if (r->host) return TYPED(init_eq, r->lattice, r->prec, *r, r->host, r->host + r->ncell, s->stream);
+    double *buf = nullptr;
+    cudaError_t e = cudaMallocAsync((void **)&buf, host_bytes(r), s->stream);
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(buf, r->pageable.data(), host_bytes(r), cudaMemcpyHostToDevice, s->stream);  // (staged by the call)
+    if (e == cudaSuccess) e = TYPED(init_eq, r->lattice, r->prec, *r, buf, buf + r->ncell, s->stream);
+    cudaFreeAsync(buf, s->stream);
+    return e;
+}
+
 // Admission: first fit in arrival order while budget and slots allow.  The
 // allocation, the initial state's upload, the equilibrium kernel and the
 // domain-table entry are enqueued on the server stream (pageable host data
-// are staged by the copy calls themselves, so nothing is awaited here).
+// are staged by the copy calls themselves, so nothing is awaited here).  A
+// request that cannot be admitted stays in the queue with its initial state.
 static int admit(lbm_server *s)
 {
     for (auto it = s->queue.begin(); it != s->queue.end();) {
@@ -467,25 +483,15 @@ static int admit(lbm_server *s)
             else
                 e = cudaMallocAsync(&r->f[1], lat, s->stream);
         }
+        if (e == cudaSuccess) e = init_request(s, r);
         if (e != cudaSuccess) {
             cudaGetLastError();
             free_request_memory(s, r);
+            if (e != cudaErrorMemoryAllocation)
+                return sfail(s, LBM_ECUDA, "admitting request %lld: %s", (long long)r->id, cudaGetErrorString(e));
             ++it;  // device memory short of the budget: try again next round
             continue;
         }
-        if (r->host) {
-            // the kernel reads the page-locked block over the host link
-            e = TYPED(init_eq, r->lattice, r->prec, *r, r->host, r->host + r->ncell, s->stream);
-        } else {
-            double *buf = nullptr;
-            e = cudaMallocAsync((void **)&buf, host_bytes(r), s->stream);
-            if (e == cudaSuccess)  // (pageable: staged by the call)
-                e = cudaMemcpyAsync(buf, r->pageable.data(), host_bytes(r), cudaMemcpyHostToDevice, s->stream);
-            if (e == cudaSuccess) e = TYPED(init_eq, r->lattice, r->prec, *r, buf, buf + r->ncell, s->stream);
-            if (buf) cudaFreeAsync(buf, s->stream);
-            std::vector<double>().swap(r->pageable);
-        }
-        if (e != cudaSuccess) return sfail(s, LBM_ECUDA, "admitting request %lld: %s", (long long)r->id, cudaGetErrorString(e));
         BatchDomain d{};
         std::memset(&d, 0, sizeof d);
         for (int a = 0; a < 3; ++a) {
@@ -516,7 +522,11 @@ static int admit(lbm_server *s)
         // admitted again, after this copy was staged
         s->doms_h[slot] = d;
         e = cudaMemcpyAsync(s->doms_d + slot, &s->doms_h[slot], sizeof(BatchDomain), cudaMemcpyHostToDevice, s->stream);
-        if (e != cudaSuccess) return sfail(s, LBM_ECUDA, "domain table upload: %s", cudaGetErrorString(e));
+        if (e != cudaSuccess) {
+            free_request_memory(s, r);
+            return sfail(s, LBM_ECUDA, "domain table upload: %s", cudaGetErrorString(e));
+        }
+        std::vector<double>().swap(r->pageable);
         s->slot_req[slot] = r->id;
         s->remaining[slot] = r->steps;
         r->slot = slot;
@@ -696,6 +706,19 @@ extern "C" int lbm_server_set_streaming(lbm_server_handle s, int pattern)
     if (pattern != LBM_STREAM_PULL && pattern != LBM_STREAM_AA)
         return sfail(s, LBM_EINVAL, "pattern must be LBM_STREAM_PULL or LBM_STREAM_AA");
     s->pattern = pattern;
+    return LBM_OK;
+}
+
+extern "C" int lbm_server_set_host_memory(lbm_server_handle s, size_t lend_bytes, size_t keep_bytes)
+{
+    if (!s) return sfail(nullptr, LBM_EINVAL, "null server");
+    s->host_lend = lend_bytes;
+    s->host_keep = keep_bytes;
+    while (s->kept > s->host_keep) {
+        cudaFreeHost(s->blocks.front().first);
+        s->kept -= s->blocks.front().second;
+        s->blocks.erase(s->blocks.begin());
+    }
     return LBM_OK;
 }
 

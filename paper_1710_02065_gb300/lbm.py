@@ -105,6 +105,7 @@ _sig("lbm_server_last_error", [C.c_void_p], C.c_char_p)
 _sig("lbm_server_submit", [C.c_void_p, C.POINTER(lbm_request), _i64p])
 _sig("lbm_server_run", [C.c_void_p, C.c_int64, _ip])
 _sig("lbm_server_set_streaming", [C.c_void_p, C.c_int])
+_sig("lbm_server_set_host_memory", [_h, C.c_size_t, C.c_size_t])
 _sig("lbm_server_set_launch", [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int])
 _sig("lbm_set_level_streams", [C.c_void_p, C.c_int])
 _sig("lbm_server_get_launch", [C.c_void_p, C.c_int, C.c_int, _ip, _ip])
@@ -487,6 +488,10 @@ def lbm_server_submit(s, lattice: int, precision: int, extents, tau: float, step
 def lbm_server_set_streaming(s, pattern: int):
     """Streaming pattern of the requests admitted from now on."""
     return _scheck(_lib.lbm_server_set_streaming(s, int(pattern)), s)
+
+
+def lbm_server_set_host_memory(s, lend_bytes: int, keep_bytes: int):
+    _scheck(_lib.lbm_server_set_host_memory(s, lend_bytes, keep_bytes), s)
 
 
 def lbm_server_set_launch(s, lattice: int, precision: int, cells_per_lane: int, warps_per_block: int):
