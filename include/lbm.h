@@ -491,7 +491,9 @@ int lbm_force(lbm_handle h, int level, double F[3]);
  *                     are device data): an index outside [0, ncell) is
  *                     skipped and its output set to NaN.
  * Both return launch errors at once and execution errors at the next
- * synchronising call.
+ * synchronising call.  A call captured into the caller's CUDA graph may be
+ * replayed after the level's cell types changed (lbm_force_async then takes the
+ * new ones), not after they were removed (lbm_set_geometry with NULL).
  */
 int lbm_force_async(lbm_handle h, int level, double *F_dev);
 int lbm_probe_async(lbm_handle h, int n, const int64_t *cells_dev, double *p_dev);

@@ -275,69 +275,92 @@ static __global__ void k_reduce_final(int nblocks, const double *__restrict__ pa
 }
 
 // Momentum-exchange force on solid cells: every fluid cell x and direction i
-// with x + xi_i solid adds 2 xi_i f*_i(x) (halfway bounce-back link).  `cells`
-// lists the fluid cells next to a solid (built by the host with the mask): a
-// scan of the whole mask for them, a second kernel for the totals and a copy
-// of the result took 17.8 us per sample of the 1600 x 800 cylinder (whose list
-// holds a few hundred cells), this one launch 8.0 us, most of it the latency
-// of its dependent loads (GB300).
+// with x + xi_i solid adds 2 xi_i f*_i(x) (halfway bounce-back link).  `near`
+// lists the fluid cells next to a solid (built by the host with the mask).  It is
+// read here, from a place that lasts as long as the level: a launch that a
+// caller captured finds the list of the geometry set last (1.3 us of the 9.3; as
+// kernel arguments the list would be one that has been freed).  A scan of the
+// whole mask for the cells, a second kernel for the totals and a copy of the
+// result took 17.8 us per sample of the 1600 x 800 cylinder (whose list holds a few
+// hundred cells), this one launch 9.3 us, most of it the latency of its dependent
+// loads (GB300).
 // Blocks are small so that the FP64 sums (two lanes per SM and cycle) spread
-// over many SMs; the block that finishes last adds the blocks' partial sums in
-// a fixed order, writes F and leaves the counter at zero for the next launch.
+// over many SMs; the block that finishes last adds the parts' sums in a fixed
+// order, writes F and leaves the counter at zero for the next launch.  The parts
+// (force_parts of the list; one per block unless the list changed after the
+// launch was captured) do not depend on the grid, so neither does F.
 constexpr int kForceBlock = 64;
+
+struct NearList {
+    const int *cells;
+    int64_t count;
+};
+
+__host__ __device__ inline int force_parts(int64_t count, int max_parts)
+{
+    const int64_t parts = (count + kForceBlock - 1) / kForceBlock;
+    return (int)(parts < max_parts ? parts : max_parts);
+}
 
 template <class L, class S>
 __global__ void __launch_bounds__(kForceBlock) k_force(int nx, int ny, int nz, int px, int py, int pz,
                                                        const S *__restrict__ f, const uint8_t *__restrict__ mask,
-                                                       const int *__restrict__ cells, int count, double *partial,
-                                                       unsigned *done, double *__restrict__ F,
+                                                       const NearList *__restrict__ near, int max_parts,
+                                                       double *partial, unsigned *done, double *__restrict__ F,
                                                        const double *__restrict__ dsh = nullptr)
 {
     const int64_t N = (int64_t)nx * ny * nz;
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (int t = blockIdx.x * kForceBlock + threadIdx.x; t < count; t += gridDim.x * kForceBlock) {
-        const int cell = cells[t];
-        const int x = cell % nx, y = (cell / nx) % ny, z = cell / (nx * ny);
-        // all mask bytes, then all populations: two rounds of loads in flight
-        // together instead of a chain of Q - 1 pairs
-        bool link[L::Q];
-        typename StoreC<S>::C v[L::Q];
-#pragma unroll
-        for (int i = 1; i < L::Q; ++i) {
-            int X = x + L::cx(i), Y = y + L::cy(i), Z = z + L::cz(i);
-            if (px) X = X < 0 ? X + nx : (X >= nx ? X - nx : X);
-            if (py) Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
-            if (pz) Z = Z < 0 ? Z + nz : (Z >= nz ? Z - nz : Z);
-            const bool in = X >= 0 && X < nx && Y >= 0 && Y < ny && Z >= 0 && Z < nz;
-            link[i] = (mask[in ? X + (int64_t)nx * (Y + (int64_t)ny * Z) : cell] & MASK_TYPE) == MASK_SOLID;  // (`cell` is fluid)
-        }
-#pragma unroll
-        for (int i = 1; i < L::Q; ++i) v[i] = Store<S>::ld(f + (int64_t)i * N + cell);
-#pragma unroll
-        for (int i = 1; i < L::Q; ++i) {
-            if (!link[i]) continue;
-            const double fi = (double)v[i] + (dsh ? dsh[i] : 0.0) + weight<L>(i);
-            if (L::cx(i)) acc[0] += L::cx(i) > 0 ? fi : -fi;
-            if (L::cy(i)) acc[1] += L::cy(i) > 0 ? fi : -fi;
-            if (L::cz(i)) acc[2] += L::cz(i) > 0 ? fi : -fi;
-        }
-    }
+    const int *__restrict__ cells = near->cells;
+    const int64_t count = near->count;
+    const int parts = force_parts(count, max_parts);
     __shared__ double sh[kForceBlock / 32][3];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int part = blockIdx.x; part < parts; part += gridDim.x) {
+        double acc[3] = {0.0, 0.0, 0.0};
+        for (int64_t t = part * kForceBlock + threadIdx.x; t < count; t += parts * kForceBlock) {
+            const int cell = cells[t];
+            const int x = cell % nx, y = (cell / nx) % ny, z = cell / (nx * ny);
+            // all mask bytes, then all populations: two rounds of loads in flight
+            // together instead of a chain of Q - 1 pairs
+            bool link[L::Q];
+            typename StoreC<S>::C v[L::Q];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        double v = 2.0 * acc[k];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) sh[warp][k] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < 3; ++k) {
-            double v = 0.0;
-            for (int w = 0; w < kForceBlock / 32; ++w) v += sh[w][k];
-            partial[3 * blockIdx.x + k] = v;
+            for (int i = 1; i < L::Q; ++i) {
+                int X = x + L::cx(i), Y = y + L::cy(i), Z = z + L::cz(i);
+                if (px) X = X < 0 ? X + nx : (X >= nx ? X - nx : X);
+                if (py) Y = Y < 0 ? Y + ny : (Y >= ny ? Y - ny : Y);
+                if (pz) Z = Z < 0 ? Z + nz : (Z >= nz ? Z - nz : Z);
+                const bool in = X >= 0 && X < nx && Y >= 0 && Y < ny && Z >= 0 && Z < nz;
+                link[i] = (mask[in ? X + (int64_t)nx * (Y + (int64_t)ny * Z) : cell] & MASK_TYPE) == MASK_SOLID;  // (`cell` is fluid)
+            }
+#pragma unroll
+            for (int i = 1; i < L::Q; ++i) v[i] = Store<S>::ld(f + (int64_t)i * N + cell);
+#pragma unroll
+            for (int i = 1; i < L::Q; ++i) {
+                if (!link[i]) continue;
+                const double fi = (double)v[i] + (dsh ? dsh[i] : 0.0) + weight<L>(i);
+                if (L::cx(i)) acc[0] += L::cx(i) > 0 ? fi : -fi;
+                if (L::cy(i)) acc[1] += L::cy(i) > 0 ? fi : -fi;
+                if (L::cz(i)) acc[2] += L::cz(i) > 0 ? fi : -fi;
+            }
         }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            double v = 2.0 * acc[k];
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) sh[warp][k] = v;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int k = 0; k < 3; ++k) {
+                double v = 0.0;
+                for (int w = 0; w < kForceBlock / 32; ++w) v += sh[w][k];
+                partial[3 * part + k] = v;
+            }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
         __threadfence();
         last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
     }
@@ -346,7 +369,7 @@ __global__ void __launch_bounds__(kForceBlock) k_force(int nx, int ny, int nz, i
     __threadfence();
     for (int k = 0; k < 3; ++k) {
         double v = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(partial + 3 * b + k);
+        for (int b = lane; b < parts; b += 32) v += __ldcg(partial + 3 * b + k);
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
         if (lane == 0) F[k] = v;
     }

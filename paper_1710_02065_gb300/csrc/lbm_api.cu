@@ -29,6 +29,7 @@ struct FineLevel {
     uint8_t *mask_d = nullptr;           // ring fixed + user solids
     bool has_solid = false;              // the mask holds solid cells
     int *near_d = nullptr;               // fluid cells next to a solid (the force's links start there)
+    NearList *list_d = nullptr;          // {near_d, nnear} for the force kernel
     int nnear = 0;
     std::vector<uint8_t> user_mask;      // user solids (host copy)
     RefineGeom geom{};                   // position in the parent level's nodes
@@ -54,6 +55,7 @@ struct lbm_ctx {
     uint8_t *solid_d = nullptr;
     bool has_solid = false;  // level 0's mask holds solid cells (else only fixed ones)
     int *near_d = nullptr;   // level 0's fluid cells next to a solid
+    NearList *list_d = nullptr;
     int nnear = 0;
     double *prof_d[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     int kind[6] = {0, 0, 0, 0, 0, 0};
@@ -131,7 +133,7 @@ struct GridRef {
     void **f;
     int *cur;
     const uint8_t *mask;
-    const int *near;  // fluid cells next to a solid
+    const NearList *list;  // fluid cells next to a solid, and their number
     int nnear;
 };
 
@@ -142,7 +144,7 @@ static const double *shift_of(const lbm_ctx *h, const GridRef &g)
 
 static GridRef coarse_ref(lbm_ctx *h)
 {
-    return GridRef{{h->n[0], h->n[1], h->n[2]}, h->ncell, h->f, &h->cur, h->solid_d, h->near_d, h->nnear};
+    return GridRef{{h->n[0], h->n[1], h->n[2]}, h->ncell, h->f, &h->cur, h->solid_d, h->list_d, h->nnear};
 }
 static int nlevels(const lbm_ctx *h) { return 1 + (int)h->levels.size(); }
 static FineLevel *fine_level(lbm_ctx *h, int k) { return h->levels[(size_t)k - 1]; }  // k >= 1
@@ -150,7 +152,7 @@ static GridRef level_grid(lbm_ctx *h, int k)
 {
     if (k == 0) return coarse_ref(h);
     FineLevel *F = fine_level(h, k);
-    return GridRef{{F->n[0], F->n[1], F->n[2]}, F->ncell, F->f, &F->cur, F->mask_d, F->near_d, F->nnear};
+    return GridRef{{F->n[0], F->n[1], F->n[2]}, F->ncell, F->f, &F->cur, F->mask_d, F->list_d, F->nnear};
 }
 static double level_tau(lbm_ctx *h, int k) { return k == 0 ? h->tau : fine_level(h, k)->tau; }
 // Bytes of one interface-moment buffer of a refined level (sized for FP64)
@@ -292,11 +294,11 @@ template <class L, class S>
 struct Force {
     // F (device, 3 doubles); partial: 3 doubles per block; done: block counter, zero between launches
     static cudaError_t run(cudaStream_t st, const int *n, const int *per, const void *f, const uint8_t *mask,
-                           const int *cells, int count, int blocks, double *partial, unsigned *done, double *F,
+                           const NearList *list, int blocks, int max_parts, double *partial, unsigned *done, double *F,
                            const double *dsh)
     {
         k_force<L, S><<<blocks, kForceBlock, 0, st>>>(n[0], n[1], n[2], per[0], per[1], per[2], (const S *)f, mask,
-                                                      cells, count, partial, done, F, dsh);
+                                                      list, max_parts, partial, done, F, dsh);
         return cudaGetLastError();
     }
 };
@@ -448,6 +450,7 @@ static void release(lbm_ctx *h)
     if (h->err_d) cudaFree(h->err_d);
     if (h->done_d) cudaFree(h->done_d);
     if (h->near_d) cudaFree(h->near_d);
+    if (h->list_d) cudaFree(h->list_d);
     if (h->chi_tab_f) cudaFree(h->chi_tab_f);
     if (h->stage_d) cudaFree(h->stage_d);
     if (h->bad_d) cudaFree(h->bad_d);
@@ -467,6 +470,7 @@ static void release(lbm_ctx *h)
         }
         if (F->mask_d) cudaFree(F->mask_d);
         if (F->near_d) cudaFree(F->near_d);
+        if (F->list_d) cudaFree(F->list_d);
         delete F;
     }
     delete h;
@@ -658,16 +662,19 @@ static int upload_level_mask(lbm_ctx *h, int k)
         if ((m[c] & MASK_TYPE) == 0 && (m[c] & MASK_NEAR_SOLID)) near.push_back((int)c);
     int *&nd = k == 0 ? h->near_d : fine_level(h, k)->near_d;
     int &nn = k == 0 ? h->nnear : fine_level(h, k)->nnear;
+    NearList *&ld = k == 0 ? h->list_d : fine_level(h, k)->list_d;
+    int *fresh = nullptr;
+    if (!ld) CUDA_TRY(h, cudaMalloc(&ld, sizeof(NearList)));
+    if (!near.empty()) {
+        CUDA_TRY(h, cudaMalloc(&fresh, sizeof(int) * near.size()));
+        CUDA_TRY(h, cudaMemcpyAsync(fresh, near.data(), sizeof(int) * near.size(), cudaMemcpyHostToDevice, h->stream));
+    }
+    const NearList list{fresh, (int64_t)near.size()};
+    CUDA_TRY(h, cudaMemcpyAsync(ld, &list, sizeof list, cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     if (nd) CUDA_TRY(h, cudaFree(nd));
-    nd = nullptr;
-    nn = 0;
-    if (!near.empty()) {
-        CUDA_TRY(h, cudaMalloc(&nd, sizeof(int) * near.size()));
-        CUDA_TRY(h, cudaMemcpyAsync(nd, near.data(), sizeof(int) * near.size(), cudaMemcpyHostToDevice, h->stream));
-        CUDA_TRY(h, cudaStreamSynchronize(h->stream));
-        nn = (int)near.size();
-    }
+    nd = fresh;
+    nn = (int)near.size();
     return LBM_OK;
 }
 
@@ -1653,16 +1660,17 @@ static int enqueue_force(lbm_ctx *h, int level, double *F_dev)
     int rc = level_ref(h, level, g);
     if (rc != LBM_OK) return rc;
     cudaError_t e;
-    if (!g.mask || g.nnear == 0) {
+    if (!g.mask) {
         e = cudaMemsetAsync(F_dev, 0, 3 * sizeof(double), h->stream);
     } else {
         int per[3] = {1, 1, 1};
         if (level == 0)
             for (int a = 0; a < 3; ++a) per[a] = h->kind[2 * a] == LBM_BC_PERIODIC ? 1 : 0;
-        const int blocks = std::min((g.nnear + kForceBlock - 1) / kForceBlock, h->red_blocks);
+        // (at least one block also for an empty list: a captured launch may find a longer one)
+        const int blocks = std::max(1, force_parts(g.nnear, h->red_blocks));
         e = dispatch<Force>(h->lattice, h->prec, h->stream, (const int *)g.n, (const int *)per,
-                            (const void *)g.f[*g.cur], g.mask, g.near, g.nnear, blocks, h->red_d, h->done_d, F_dev,
-                            shift_of(h, g));
+                            (const void *)g.f[*g.cur], g.mask, g.list, blocks, h->red_blocks, h->red_d,
+                            h->done_d, F_dev, shift_of(h, g));
         h->launches += 1;
     }
     if (e != cudaSuccess) return fail(h, LBM_ECUDA, "force: %s", cudaGetErrorString(e));
