@@ -239,9 +239,17 @@ static double *take_block(lbm_server *s, size_t bytes)
         size = best->second;
         s->kept -= size;
         s->blocks.erase(best);
-    } else if (cudaHostAlloc((void **)&b, bytes, cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    } else {
+        // a submit may come while the caller captures a graph, also in the
+        // modes that forbid allocation calls: this one has no part in it
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+        const cudaError_t e = cudaHostAlloc((void **)&b, bytes, cudaHostAllocDefault);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
     }
     s->held[b] = size;
     s->held_bytes += size;

@@ -106,3 +106,26 @@ def test_request_without_device_memory_for_its_upload_stays_queued():
     torch.cuda.synchronize()
     assert cu.cuMemPoolDestroy(pool) == 0
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+def test_submit_while_the_caller_captures_a_graph():
+    """A submit between the caller's captured launches neither fails nor ends
+    the capture, and its request is served."""
+    from paper_1710_02065_gb300 import lbm
+    n = (64, 48, 1)
+    rho, u = _state(n, 1)
+    s = lbm.lbm_server_create(1 << 28, 8)
+    x = torch.zeros(16, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="global"):
+        x += 1
+        ids = [lbm.lbm_server_submit(s, 0, lbm.LBM_FP32, n, 0.7, 20, rho, u)]
+        x += 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert (x == 2).all()
+    ids.append(lbm.lbm_server_submit(s, 0, lbm.LBM_FP32, n, 0.7, 20, rho, u))
+    a, b = _collect(s, ids, [64 * 48] * 2)
+    lbm.lbm_server_destroy(s)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
