@@ -28,12 +28,12 @@
 #include <cstring>
 #include <deque>
 #include <map>
+#include <new>
 #include <string>
-#include <system_error>
-#include <thread>
 #include <utility>
 #include <vector>
 
+#include "host_pool.h"
 #include "lbm.h"
 #include "aux_kernels.cuh"
 #include "dispatch.h"
@@ -272,30 +272,6 @@ static void return_block(lbm_server *s, double *b)
     s->kept += size;
 }
 
-// Copy between host buffers; large ones by four threads (one core's copy rate
-// is a fraction of the memory's)
-static void copy_host(double *dst, const double *src, size_t n)
-{
-    constexpr size_t kPart = size_t(1) << 18;  // doubles a thread is worth starting for
-    const size_t parts = std::min<size_t>(4, n / kPart);
-    if (parts < 2) {
-        std::memcpy(dst, src, n * sizeof(double));
-        return;
-    }
-    std::vector<std::thread> th;
-    try {
-        for (size_t k = 1; k < parts; ++k) {
-            const size_t a = n * k / parts, b = n * (k + 1) / parts;
-            th.emplace_back([=] { std::memcpy(dst + a, src + a, (b - a) * sizeof(double)); });
-        }
-    } catch (const std::system_error &) {  // no thread to be had: the rest here
-        const size_t a = n * (th.size() + 1) / parts;
-        std::memcpy(dst + a, src + a, (n - a) * sizeof(double));
-    }
-    std::memcpy(dst, src, n / parts * sizeof(double));
-    for (std::thread &t : th) t.join();
-}
-
 static int sfail(lbm_server *s, int code, const char *fmt, ...)
 {
     char buf[512];
@@ -431,7 +407,16 @@ extern "C" int lbm_server_submit(lbm_server_handle s, const lbm_request *req, in
     }
     const size_t N = (size_t)r->ncell;
     if (s->held_bytes + host_bytes(r) <= s->host_lend) r->host = take_block(s, host_bytes(r));
-    if (!r->host) r->pageable.resize(4 * N);
+    try {
+        if (!r->host) r->pageable.resize(4 * N);
+        s->reqs[s->next_id] = r;
+        s->queue.push_back(r);
+    } catch (const std::bad_alloc &) {
+        s->reqs.erase(s->next_id);
+        return_block(s, r->host);
+        delete r;
+        return sfail(s, LBM_ENOMEM, "no host memory for a request of %zu cells", N);
+    }
     double *h = r->host ? r->host : r->pageable.data();
     if (req->rho)
         copy_host(h, req->rho, N);
@@ -442,8 +427,6 @@ extern "C" int lbm_server_submit(lbm_server_handle s, const lbm_request *req, in
     else
         std::fill(h + N, h + 4 * N, 0.0);
     r->id = s->next_id++;
-    s->reqs[r->id] = r;
-    s->queue.push_back(r);
     *id = r->id;
     return LBM_OK;
 }
