@@ -1042,16 +1042,12 @@ extern "C" int lbm_get_populations(lbm_handle h, double *f)
 // ---------------------------------------------------------------------------
 // Time stepping
 // ---------------------------------------------------------------------------
-static int build_params(lbm_ctx *h, StepParams &p)
+static void fill_params(lbm_ctx *h, StepParams &p)
 {
     std::memset(&p, 0, sizeof p);
     for (int a = 0; a < 3; ++a) {
         p.n[a] = h->n[a];
-        const bool plo = h->kind[2 * a] == LBM_BC_PERIODIC, phi = h->kind[2 * a + 1] == LBM_BC_PERIODIC;
-        if (plo != phi)
-            return fail(h, LBM_EINVAL, "axis %d: both faces must be periodic or neither", a);
-        p.periodic[a] = plo ? 1 : 0;
-        if (!plo && h->n[a] < 3) return fail(h, LBM_EINVAL, "axis %d: a non-periodic axis needs >= 3 cells", a);
+        p.periodic[a] = h->kind[2 * a] == LBM_BC_PERIODIC ? 1 : 0;
     }
     p.ncell = h->ncell;
     for (int f = 0; f < 6; ++f) {
@@ -1100,6 +1096,18 @@ static int build_params(lbm_ctx *h, StepParams &p)
                         ? 1
                         : 0;
     set_bulk_box(p);
+}
+
+// The same for a step: refused while the faces do not form a lattice
+static int build_params(lbm_ctx *h, StepParams &p)
+{
+    for (int a = 0; a < 3; ++a) {
+        const bool plo = h->kind[2 * a] == LBM_BC_PERIODIC, phi = h->kind[2 * a + 1] == LBM_BC_PERIODIC;
+        if (plo != phi)
+            return fail(h, LBM_EINVAL, "axis %d: both faces must be periodic or neither", a);
+        if (!plo && h->n[a] < 3) return fail(h, LBM_EINVAL, "axis %d: a non-periodic axis needs >= 3 cells", a);
+    }
+    fill_params(h, p);
     return LBM_OK;
 }
 
@@ -1805,15 +1813,10 @@ extern "C" int lbm_set_launch(lbm_handle h, int block, int cells_per_thread)
 extern "C" int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread)
 {
     CHECK_HANDLE(h);
-    int vec = h->vec;
-    if (vec == 0) {  // the default: what level 0 runs as configured now
-        StepParams p;
-        const int rc = build_params(h, p);
-        if (rc != LBM_OK) return rc;
-        vec = pick_vec(h, p);
-    } else if (h->solid_d || !vec_available(h, vec) || h->n[0] % vec != 0) {
-        vec = 1;
-    }
+    StepParams p;  // (of level 0 as configured so far, complete or not)
+    fill_params(h, p);
+    if (h->vec > 1) p.sponge_rest = 1;  // (an explicit shape: whatever state the sponges relax to)
+    const int vec = pick_vec(h, p);
     if (block) *block = h->block > 0 ? h->block : block_default(vec, h->n[0]);  // level 0
     if (cells_per_thread) *cells_per_thread = vec;
     return LBM_OK;
