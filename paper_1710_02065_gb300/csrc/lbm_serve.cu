@@ -186,6 +186,7 @@ struct lbm_server {
     std::vector<BatchTile> tiles_h[NGROUPS];
     BatchTile *tiles_d[NGROUPS] = {};
     size_t tiles_cap[NGROUPS] = {};
+    int64_t cells_h[NGROUPS] = {};       // cells of the domains in the list
     // streams of the groups' chains within a round (the first chain runs on
     // `stream`), created when a round first needs them
     cudaStream_t side[NGROUPS] = {};
@@ -193,7 +194,7 @@ struct lbm_server {
     bool dirty = true;                   // composition changed since the graph was captured
     cudaGraphExec_t graph = nullptr;
     int64_t graph_steps = 0;
-    int sms = 152;
+    int sms = 152, l2_bytes = 129 << 20;
     // launch shape per (lattice, precision): cells per lane (0: the default
     // rule) and warps per block
     int lanes[NKINDS] = {};
@@ -327,6 +328,9 @@ extern "C" int lbm_server_create(lbm_server_handle *out, size_t hbm_budget_bytes
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
     if (sms > 0) s->sms = sms;
+    int l2 = 0;
+    cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, 0);
+    if (l2 > 0) s->l2_bytes = l2;
     *out = s;
     return LBM_OK;
 }
@@ -543,13 +547,18 @@ static int lanes_of(const lbm_server *s, const Request *r)
 // Warp tile lists per group: 32 x V consecutive cells of a row each.
 static int build_tiles(lbm_server *s)
 {
-    for (int g = 0; g < NGROUPS; ++g) s->tiles_h[g].clear();
+    for (int g = 0; g < NGROUPS; ++g) {
+        s->tiles_h[g].clear();
+        s->cells_h[g] = 0;
+    }
     for (int k = 0; k < s->max_slots; ++k) {
         if (!s->slot_req[k] || s->remaining[k] <= 0) continue;
         Request *r = s->reqs[s->slot_req[k]];
         const int v = lanes_of(s, r);
         const int segs = (r->n[0] + 32 * v - 1) / (32 * v);
-        std::vector<BatchTile> &list = s->tiles_h[group_of(r->lattice, r->prec, v, r->aa)];
+        const int g = group_of(r->lattice, r->prec, v, r->aa);
+        std::vector<BatchTile> &list = s->tiles_h[g];
+        s->cells_h[g] += r->ncell;
         for (int z = 0; z < r->n[2]; ++z)
             for (int y = 0; y < r->n[1]; ++y)
                 for (int xs = 0; xs < segs; ++xs) list.push_back(BatchTile{k, y, z, xs * 32 * v});
@@ -588,9 +597,11 @@ static cudaError_t enqueue_steps(lbm_server *s, int64_t steps)
     for (size_t k = 0; k < groups.size() && e == cudaSuccess; ++k) {
         const int g = groups[k];
         const int n = (int)s->tiles_h[g].size();
-        // persistent grid: at most 32 resident warps per SM asked for
-        const int wpb = s->wpb[g >> 2];
-        const int blocks = (n + wpb - 1) / wpb, cap = s->sms * (32 / wpb);
+        // persistent grid
+        const int wpb = s->wpb[g >> 2], kind = g >> 2;
+        const int warps = batch_warps_per_sm(kind / 4 == LBM_D3Q19, elem_bytes(kind % 4), (g & 1) + 1, (g & 2) != 0,
+                                             s->cells_h[g], n, s->l2_bytes);
+        const int blocks = (n + wpb - 1) / wpb, cap = s->sms * ((warps + wpb - 1) / wpb);
         BatchLaunch b{s->doms_d, s->tiles_d[g], n, blocks < cap ? blocks : cap, wpb, 0, k ? s->side[g] : s->stream};
         if (k) e = cudaStreamWaitEvent(b.st, s->fork_ev, 0);
         for (int64_t t = 0; t < steps && e == cudaSuccess; ++t) {

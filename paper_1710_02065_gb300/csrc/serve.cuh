@@ -15,6 +15,8 @@
 // k_batch_advance does it once at the end of the round.
 #pragma once
 
+#include <algorithm>
+
 #include "step_vec.cuh"
 
 namespace rr {
@@ -40,12 +42,32 @@ struct BatchTile {
 
 // Resident 256-thread blocks per SM asked of the compiler: as the
 // single-lattice kernel, 16-bit storage with two cells per lane is latency-
-// bound and gets 64 registers (32 resident warps per SM) on D2Q9 / D3Q19;
+// bound and gets 64 registers (32 resident warps per SM) on D2Q9 / D3Q19, 80
+// for the in-place steps of D3Q19, whose two step types spill 180 bytes at 64;
 // the other groups keep the registers they need.
-template <class L, class S, int V>
+template <class L, class S, int V, bool AA>
 struct BatchMinBlocks {
-    static constexpr int value = (sizeof(S) == 2 && V == 2 && L::Q <= 19) ? 4 : 0;
+    static constexpr int value = (sizeof(S) == 2 && V == 2 && L::Q <= 19) ? (AA && L::Q == 19 ? 3 : 4) : 0;
 };
+
+// Warps per SM that a group's persistent grid asks for: 32, as many as can be
+// resident, unless more rows at a time cost more in the caches than their
+// latency hides.  GB300, G cell updates/s, two cells per lane, by warps per SM:
+//   D3Q19 FP32 pull, 8 x 128^3 32 40.2, 24 40.4, 20 40.5, 16 41.1, 14 42.8, 12 44.6,
+//     10 41.3; rows that fill their last tile in part are best with as many
+//     cells at a time: 160^3 (0.83 full) 32 37.4, 16 41.1, 14 41.7, 12 39.6, 8 x 96^3
+//     (0.75 full) 32 38.8, 16 42.5, 12 38.2.  A group within twice the L2's bytes
+//     does not gain: 4 x 64^3 (159 MB) 32 43.8, 12 39.9, 1 x 128^3 (319 MB) 38.5, 41.6.
+//   D3Q19 FP16 in place (80 registers), a batch of 60^3 to 128^3 32 56.5, 24 64.4,
+//     20 62.8, 16 58.8 (at 64 registers 55.9 to 58.1, at 100 60.8).
+// cells, tiles: of the group's domains; its lattices' bytes are elem 2 Q cells.
+inline int batch_warps_per_sm(bool d3q19, size_t elem, int v, bool aa, int64_t cells, int64_t tiles, int64_t l2_bytes)
+{
+    if (!d3q19 || v != 2) return 32;
+    if (aa) return elem == 2 ? 24 : 32;
+    if (elem != 4 || 2 * 19 * 4 * cells <= 2 * l2_bytes) return 32;
+    return (int)std::min<int64_t>(32, (12 * 64 * tiles + cells / 2) / cells);
+}
 
 // V cells of a row of a fully periodic domain, all of them bulk cells: the
 // vector update of step_vec.cuh without its boundary roles.  Compiled for one
@@ -132,7 +154,7 @@ __device__ __forceinline__ void update_served(const BatchDomain &d, const char *
 // Step s of a round for the domains of one group.  tiles: the group's list;
 // the next item is fetched while the current one is updated.
 template <class L, class S, class C, int V, bool AA>
-__global__ void __launch_bounds__(256, (BatchMinBlocks<L, S, V>::value))
+__global__ void __launch_bounds__(256, (BatchMinBlocks<L, S, V, AA>::value))
     k_batched(const BatchDomain *__restrict__ doms, const int4 *__restrict__ tiles, int ntiles, int s)
 {
     const int wpb = blockDim.x >> 5, lane = threadIdx.x & 31;
