@@ -303,9 +303,9 @@ int lbm_probe(lbm_handle h, int n, const int64_t *cells, double *p_prime);
  *                      run when the row-staged kernel (lbm_set_staging) is off
  *                      or not eligible.
  * lbm_get_launch reports the shape lbm_step will use on level 0 as the handle
- * is configured now, complete or not.  (An explicitly set shape is reported
- * also while sponges relax to another state than rest, where the general
- * kernel runs instead.)
+ * is configured now, complete or not.  An explicitly set shape is reported as
+ * set also under plain BGK, order 4 and sponges that the vectorised kernel does
+ * not take, where the general kernel runs instead.
  */
 int lbm_set_launch(lbm_handle h, int block, int cells_per_thread);
 int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread);

@@ -1815,7 +1815,8 @@ extern "C" int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread)
     CHECK_HANDLE(h);
     StepParams p;  // (of level 0 as configured so far, complete or not)
     fill_params(h, p);
-    if (h->vec > 1) p.sponge_rest = 1;  // (an explicit shape: whatever state the sponges relax to)
+    // an explicit shape is reported whatever collision and sponges are selected
+    if (h->vec > 1) p.bgk = p.order4 = p.any_sponge = 0;
     const int vec = pick_vec(h, p);
     if (block) *block = h->block > 0 ? h->block : block_default(vec, h->n[0]);  // level 0
     if (cells_per_thread) *cells_per_thread = vec;
