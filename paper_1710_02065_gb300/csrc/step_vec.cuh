@@ -492,10 +492,12 @@ __device__ __forceinline__ void add_shift(const StepParams &p, C *g, C sign)
 // its sponge strength from the per-axis tables (0 in the bulk) and the
 // closed-form coefficients of a rest-state reference.  A node on a
 // non-periodic x face collides its neighbour's streamed populations: as they
-// are (outflow face) or with the face's density / velocity substituted.
+// are (outflow face) or with the face's density / velocity substituted; so do
+// the nodes of a row on the face row_inlet (>= 0, 2D).
 template <class L, class S, class C, int V, int G, int SP, int WR, bool SH>
 __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out0, int x0, int y, int z,
-                                                  const RowOff &ro, const VecIn<L, S, C, V> &r, bool all_bulk)
+                                                  const RowOff &ro, const VecIn<L, S, C, V> &r, bool all_bulk,
+                                                  int row_inlet)
 {
     const int nx = p.n[0];
     const unsigned nxy = (unsigned)nx * (unsigned)p.n[1];
@@ -531,8 +533,8 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
                 add_shift<L, C, SH>(p, g, C(1));
                 m = moments_pairs<L, C>(g);
                 const int x = x0 + k;
-                const int inlet = !face ? -1 : (k == 0 ? (p.kind[0] != BC_OUTFLOW ? 0 : -1)
-                                                        : (p.kind[1] != BC_OUTFLOW ? 1 : -1));
+                int inlet = row_inlet;  // (an x face comes before the row's)
+                if (face && p.kind[k == 0 ? 0 : 1] != BC_OUTFLOW) inlet = k == 0 ? 0 : 1;
                 if (inlet >= 0) {
                     m = face_moments<L, C>(p, m, inlet, x, y, z);
                 } else {
@@ -558,28 +560,35 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
     }
 }
 
-// Whether the vector path applies to row (y, z), and the row sy whose streamed
-// populations it collides.  3D: rows whose y / z neighbour rows do not wrap and
+// Whether the vector path applies to row (y, z), the row sy whose streamed
+// populations it collides and the face whose density / velocity they take
+// (inlet, -1: none).  3D: rows whose y / z neighbour rows do not wrap and
 // that are not on a non-periodic y / z face (for the AA steps, nor next to
-// one).  2D: the rows of a periodic y axis, wrapped around, and for the pull
-// also outflow face rows, which take the inward neighbour row's populations
-// as they are.  The other rows run the general update, V cells one after the
-// other.  (In 2D that took 1.0 us of a 1024 x 1024 FP16 step, 7.96 -> 6.95 us:
-// two rows, but they finish last; the 3D kernels lost 2 % at 384 x 256 x 256 to
-// the offsets that these rows need.)  The handle's sponge layers
-// relax to the rest state (the vector path's closed form) -- launch_update
-// checks it.
+// one).  2D: for the pull every row -- those of a periodic y axis wrapped
+// around, face rows with the inward neighbour row's populations -- and for the AA
+// steps all but face rows and the rows next to one.  The other rows run the
+// general update, V cells one after the other.  (Two rows, but they finish last.
+// GB300, us per step with / without the general update there: D2Q9 FP16
+// 1024 x 1024 periodic 7.96 / 6.95; between free-slip walls FP32 128 x 128
+// 2.70 / 1.93 (one cell per thread 1.86), 400 x 200 3.12 / 2.32 (2.43), 1024 x 1024
+// 8.88 / 8.08 (9.58).  The 3D kernels lost 2 % at 384 x 256 x 256 to the offsets that
+// these rows need.)  The handle's sponge layers relax to the rest state (the
+// vector path's closed form) -- launch_update checks it.
 template <class L, int SP>
-__device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z, int &sy)
+__device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z, int &sy, int &inlet)
 {
     const int ny = p.n[1], nz = p.n[2];
     sy = y;
+    inlet = -1;
     bool ok = p.off32 && !p.order4;
     if constexpr (L::D == 2) {
         if (p.periodic[1]) return ok;
         if (SP != kPull) return ok && y > 1 && y < ny - 2;
-        if (y == 0) { sy = 1; ok = ok && p.kind[2] == BC_OUTFLOW; }
-        if (y == ny - 1) { sy = y - 1; ok = ok && p.kind[3] == BC_OUTFLOW; }
+        if (y == 0 || y == ny - 1) {
+            sy = y == 0 ? 1 : ny - 2;
+            const int face = y == 0 ? 2 : 3;
+            if (p.kind[face] != BC_OUTFLOW) inlet = face;
+        }
         return ok;
     }
     ok = ok && y > 0 && y < ny - 1 && z > 0 && z < nz - 1;
@@ -618,14 +627,14 @@ __device__ __forceinline__ void update_vec(const StepParams &p, const char *cons
 {
     const int nx = p.n[0];
     if (x0 >= nx) return;  // lanes past the row end
-    int sy = y;
-    if (WR || vec_row<L, SP>(p, y, z, sy)) {
+    int sy = y, inlet = -1;
+    if (WR || vec_row<L, SP>(p, y, z, sy, inlet)) {
         const RowOff ro = row_offsets<L, WR>(p, sy, z);
         VecIn<L, S, C, V> r;
         if (!vec_load<L, S, C, V, SP, CH>(p, in[0], x0, sy, z, ro, r)) return;
         const bool bulk = y >= p.blo[1] && y < p.bhi[1] && z >= p.blo[2] && z < p.bhi[2] && x0 >= p.blo[0] &&
                           x0 + V <= p.bhi[0];
-        vec_collide_store<L, S, C, V, G, SP, WR, SH>(p, out[0], x0, y, z, ro, r, bulk);
+        vec_collide_store<L, S, C, V, G, SP, WR, SH>(p, out[0], x0, y, z, ro, r, bulk, L::D == 2 ? inlet : -1);
         return;
     }
     if constexpr (!WR) {
