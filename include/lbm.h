@@ -291,8 +291,9 @@ int lbm_probe(lbm_handle h, int n, const int64_t *cells, double *p_prime);
  *   cells_per_thread : 1 = one cell per thread (the general kernel); 2 or 4 =
  *                      vectorised kernel with that many consecutive x cells per
  *                      thread (FP64: 2; FP32, FP16, BF16: 2 or 4); 0 = default
- *                      (measured fastest on GB300: 1 for FP64 and for FP32
- *                      on D3Q19, else 2).  The vectorised kernel is used only
+ *                      (measured fastest on GB300: 1 for FP64, for FP32 on
+ *                      D3Q19 and for small in-place D2Q9 lattices that are not
+ *                      periodic in y, else 2).  The vectorised kernel is used only
  *                      when nx is a multiple of it (on D3Q27 only with 2 cells
  *                      per thread), a direction's arrays span less than 2 GB in
  *                      all, and there is no cell-type mask, fourth order or

@@ -74,6 +74,13 @@ inline int vec_default(int lattice, int precision)
     if (precision == PREC_FP32) return lattice == 1 /* D3Q19 */ ? 1 : 2;
     return 2;
 }
+// Small D2Q9 lattices whose in-place steps run one cell per thread by default
+// when the y axis is not periodic: the two rows next to its faces take the general
+// update, in the vectorised kernel V cells one after the other, and finish last.
+// GB300, us per step, one cell / two (inlet, outflow on the other faces): FP32
+// 128^2 4.12 / 5.57, 512^2 6.87 / 7.38, 700 x 400 7.19 / 7.69, 1024 x 512 9.95 / 9.14;
+// FP16 128^2 4.23 / 5.38, 256^2 4.55 / 5.64, 512^2 7.09 / 6.77.
+inline bool aa_small_2d(int64_t ncell, size_t elem) { return ncell <= (int64_t)elem << 16; }
 // Default threads per block.  The vectorised kernel's blocks lie along x
 // rows of nx / vec threads, so the block has to divide the row's warps or the
 // last block of every row holds idle warps: 64 threads where the row is a

@@ -1134,7 +1134,8 @@ static bool vec_eligible(const lbm_ctx *h, const StepParams &p, int vec)
 // number where the vectorised kernel can run it, else 1 (the general kernel)
 static int pick_vec(const lbm_ctx *h, const StepParams &p)
 {
-    const int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
+    int vec = h->vec == 0 ? vec_default(h->lattice, h->prec) : h->vec;
+    if (h->vec == 0 && h->pattern == LBM_STREAM_AA && h->d == 2 && !p.periodic[1] && aa_small_2d(p.ncell, h->elem)) vec = 1;
     // (the vector path addresses a lattice with 32-bit offsets)
     const bool off32 = (int64_t)h->q * p.ncell * (int64_t)h->elem < ((int64_t)1 << 31);
     return vec > 1 && p.n[0] % vec == 0 && off32 && vec_available(h, vec) && vec_eligible(h, p, vec) ? vec : 1;

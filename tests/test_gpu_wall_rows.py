@@ -89,3 +89,29 @@ def test_default_shape_between_walls_is_not_the_slower_one(prec, n):
     quarter for timing and the edges' longer code (it was 1.2 to 1.45 times)."""
     kinds = (VELOCITY, OUTFLOW, FREESLIP, FREESLIP)
     assert step_us(n, prec, kinds, False, 0) < 1.25 * step_us(n, prec, kinds, False, 1)
+
+
+@pytest.mark.parametrize("prec,n,cells", [("fp32", (512, 512, 1), 1), ("fp32", (512, 514, 1), 2), ("fp16", (512, 256, 1), 1),
+                                          ("bf16", (512, 258, 1), 2), ("fp32", (64, 6, 1), 1)])
+@pytest.mark.parametrize("walls", [True, False])
+def test_small_in_place_lattices_take_one_cell_per_thread(prec, n, cells, walls):
+    """At the edges of the rule; a periodic y axis keeps two, as does the pull."""
+    from paper_1710_02065_gb300 import lbm
+    s = lbm.Solver(D2Q9, n, 0.6, PRECS[prec])
+    for face in (2, 3) if walls else ():
+        lbm.lbm_set_boundary(s.h, face, FREESLIP)
+    assert lbm.lbm_get_launch(s.h)[1] == 2
+    lbm.lbm_set_streaming(s.h, lbm.LBM_STREAM_AA)
+    assert lbm.lbm_get_launch(s.h)[1] == (cells if walls else 2)
+    lbm.lbm_set_launch(s.h, 0, 2)
+    assert lbm.lbm_get_launch(s.h)[1] == 2
+    s.close()
+
+
+@pytest.mark.parametrize("n", [(128, 128, 1), (400, 200, 1)])
+@pytest.mark.parametrize("prec", ["fp32", "fp16"])
+def test_default_in_place_shape_is_not_the_slower_one(prec, n):
+    """The default against one cell per thread, with a tenth for timing (it was
+    1.2 to 1.35 times)."""
+    kinds = (VELOCITY, OUTFLOW, OUTFLOW, OUTFLOW)
+    assert step_us(n, prec, kinds, True, 0) < 1.1 * step_us(n, prec, kinds, True, 1)
