@@ -561,10 +561,18 @@ __device__ __forceinline__ void cell_collide(const StepParams &p, const Mom<C> &
 // HBM.  GB300, us per pass without / with it: D2Q9 FP64 128^2 pulse 946 / 883, two-
 // level D2Q9 FP32 cylinder 1511 / 1483, cylinder 3407 / 3373, D3Q27 FP16 jet (the
 // rows at y and z faces) 4874 / 4746; the HBM-bound D3Q19 FP32 jet 28320 / 28548.
+// The loads of 3D 16-bit storage only in rows without x faces: a warp at an x
+// sponge runs both forms (161 x 129 x 97 open box, us per step with / without:
+// D3Q19 FP16 39.9 / 39.1, D3Q27 FP16 56.7 / 55.1; 95 x 64 x 64 D3Q27 FP16 13.0 / 12.4).
 template <class L, class S>
 __host__ __device__ constexpr bool uniform_rows()
 {
     return L::D == 2 || sizeof(S) != 4;
+}
+template <class L, class S>
+__device__ __forceinline__ bool uniform_loads(const StepParams &p)
+{
+    return uniform_rows<L, S>() && p.off32 && (L::D == 2 || sizeof(S) == 8 || p.periodic[0]);
 }
 
 template <class L, class S, class C, bool BGK = false, int MASK = kMaskLinks, bool CH = false>
@@ -638,7 +646,7 @@ __device__ __forceinline__ void update_cell(const StepParams &p, const char *con
             if (p.shifted) g[i] += dsh<C>(p, k);
         }
     } else {
-        if (uniform_rows<L, S>() && p.off32 && bulk && (unsigned)(y - 1) < ny - 2 && (L::D == 2 || (unsigned)(z - 1) < nz - 2)) {
+        if (uniform_loads<L, S>(p) && bulk && (unsigned)(y - 1) < ny - 2 && (L::D == 2 || (unsigned)(z - 1) < nz - 2)) {
             // rows that do not wrap: each direction's row is a fixed distance from
             // the cell's, the same for every thread, so the addresses are three
             // 32-bit offsets (x, x - 1, x + 1) on uniform bases
