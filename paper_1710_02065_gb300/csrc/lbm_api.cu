@@ -1308,12 +1308,13 @@ static cudaError_t launch_level_2d(lbm_ctx *h, const StepParams &p, int k, int s
     q.omega_up = 1.0 - 1.0 / tau_p;
     const void *fin = F->f[F->cur];
     void *fout = F->f[1 - F->cur];
+    const int block = h->block > 0 ? h->block : kLevelBlock;
     h->launches += 1;
     switch (h->prec) {
-    case LBM_FP64: return launch_level_step_2d<double>(p, q, fin, fout, h->stream);
-    case LBM_FP32: return launch_level_step_2d<float>(p, q, fin, fout, h->stream);
-    case LBM_FP16_SHIFTED: return launch_level_step_2d<__half>(p, q, fin, fout, h->stream);
-    case LBM_BF16_SHIFTED: return launch_level_step_2d<__nv_bfloat16>(p, q, fin, fout, h->stream);
+    case LBM_FP64: return launch_level_step_2d<double>(p, q, fin, fout, block, h->stream);
+    case LBM_FP32: return launch_level_step_2d<float>(p, q, fin, fout, block, h->stream);
+    case LBM_FP16_SHIFTED: return launch_level_step_2d<__half>(p, q, fin, fout, block, h->stream);
+    case LBM_BF16_SHIFTED: return launch_level_step_2d<__nv_bfloat16>(p, q, fin, fout, block, h->stream);
     }
     return cudaErrorInvalidValue;
 }

@@ -195,7 +195,7 @@ __device__ inline void ring_coord(int nfx, int nfy, int t, int &i, int &j)
 }
 __host__ __device__ inline int ring_count(int nfx, int nfy) { return 2 * nfx + 2 * (nfy - 2); }
 
-constexpr int kLevelBlock = 128;
+constexpr int kLevelBlock = 128;  // default threads per block (lbm_set_launch)
 
 template <class S>
 __device__ __forceinline__ void level_line(const LevelStep2D &q, int e)
@@ -286,40 +286,41 @@ __device__ __forceinline__ void level_restrict(const LevelStep2D &q, int lane_id
 }
 
 template <class S, int MASK>
-__global__ void __launch_bounds__(kLevelBlock)
+__global__ void __launch_bounds__(256)
     k_level_step_2d(const __grid_constant__ StepParams p, const __grid_constant__ LevelStep2D q)
 {
     using C = CT<S>;
     int b = blockIdx.x;
-    const int tid = threadIdx.x;
-    if (b < q.nline) return level_line<S>(q, b * kLevelBlock + tid);
+    const int tid = threadIdx.x, nt = blockDim.x;
+    if (b < q.nline) return level_line<S>(q, b * nt + tid);
     b -= q.nline;
-    if (b < q.nring) return level_ring<S>(q, b * kLevelBlock + tid, (S *)p.out[0]);
+    if (b < q.nring) return level_ring<S>(q, b * nt + tid, (S *)p.out[0]);
     b -= q.nring;
-    if (b < q.nrestrict) return level_restrict<S>(q, b * kLevelBlock + tid, (const S *)p.in[0]);
+    if (b < q.nrestrict) return level_restrict<S>(q, b * nt + tid, (const S *)p.in[0]);
     b -= q.nrestrict;
-    const unsigned t = (unsigned)b * kLevelBlock + tid;
+    const unsigned t = (unsigned)b * nt + tid;
     if (t >= (unsigned)p.ncell) return;
     const unsigned nx = p.n[0], y = t / nx;
     update_cell<D2Q9, S, C, false, MASK>(p, p.in, p.out, (int)(t - y * nx), (int)y, 0);
 }
 
-// Launch one substep of a refined 2D level (fin read, fout written)
+// Launch one substep of a refined 2D level (fin read, fout written; block: a multiple of 32 up to 256)
 template <class S>
-cudaError_t launch_level_step_2d(const StepParams &p, const LevelStep2D &q0, const void *fin, void *fout, cudaStream_t st)
+cudaError_t launch_level_step_2d(const StepParams &p, const LevelStep2D &q0, const void *fin, void *fout, int block,
+                                 cudaStream_t st)
 {
     StepParams s = p;
     set_bases<D2Q9, S>(s, fin, fout);
     LevelStep2D q = q0;
-    auto blocks = [](int64_t threads) { return (int)((threads + kLevelBlock - 1) / kLevelBlock); };
+    auto blocks = [block](int64_t threads) { return (int)((threads + block - 1) / block); };
     q.nline = q.first ? blocks(line_count(q.g)) : 0;
     q.nring = blocks(4 * (int64_t)ring_count(q.g.nfx, q.g.nfy));
     q.nrestrict = q.first ? 0 : blocks(16 * (int64_t)ring_count(q.g.Wc - 1, q.g.Hc - 1));
     const unsigned grid = (unsigned)(q.nline + q.nring + q.nrestrict + blocks(p.ncell));
     if (p.any_solid)
-        k_level_step_2d<S, kMaskLinks><<<grid, kLevelBlock, 0, st>>>(s, q);
+        k_level_step_2d<S, kMaskLinks><<<grid, block, 0, st>>>(s, q);
     else
-        k_level_step_2d<S, kMaskSkip><<<grid, kLevelBlock, 0, st>>>(s, q);
+        k_level_step_2d<S, kMaskSkip><<<grid, block, 0, st>>>(s, q);
     return cudaGetLastError();
 }
 
