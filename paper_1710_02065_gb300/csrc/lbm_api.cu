@@ -650,16 +650,24 @@ static int upload_level_mask(lbm_ctx *h, int k)
                 for (int x = c.X0 + 1; x < c.X0 + c.Wc; ++x) at(x, y, z) = LBM_CELL_FIXED;
     }
     add_near_solid(h, m, g.n);
+    // whether there are solids, and the fluid cells next to one, for the force;
+    // eight cells at a time (most are fluid away from solids: zero)
     bool any = false;
-    for (const uint8_t v : m) any = any || (v & MASK_TYPE) == MASK_SOLID;
+    std::vector<int> near;
+    for (size_t c0 = 0; c0 < m.size(); c0 += 8) {
+        const size_t c1 = std::min(m.size(), c0 + 8);
+        uint64_t word = 0;
+        std::memcpy(&word, m.data() + c0, c1 - c0);
+        if (word == 0) continue;
+        for (size_t c = c0; c < c1; ++c) {
+            if ((m[c] & MASK_TYPE) == MASK_SOLID) any = true;
+            if ((m[c] & MASK_TYPE) == 0 && (m[c] & MASK_NEAR_SOLID)) near.push_back((int)c);
+        }
+    }
     (k == 0 ? h->has_solid : fine_level(h, k)->has_solid) = any;
     uint8_t *&dst = k == 0 ? h->solid_d : fine_level(h, k)->mask_d;
     if (!dst) CUDA_TRY(h, cudaMalloc(&dst, (size_t)g.ncell));
     CUDA_TRY(h, cudaMemcpyAsync(dst, m.data(), (size_t)g.ncell, cudaMemcpyHostToDevice, h->stream));
-    // the fluid cells next to a solid, for the force
-    std::vector<int> near;
-    for (size_t c = 0; c < m.size(); ++c)
-        if ((m[c] & MASK_TYPE) == 0 && (m[c] & MASK_NEAR_SOLID)) near.push_back((int)c);
     int *&nd = k == 0 ? h->near_d : fine_level(h, k)->near_d;
     int &nn = k == 0 ? h->nnear : fine_level(h, k)->nnear;
     NearList *&ld = k == 0 ? h->list_d : fine_level(h, k)->list_d;
