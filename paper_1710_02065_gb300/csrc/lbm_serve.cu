@@ -160,6 +160,23 @@ cudaError_t domain_offsets(StepParams &p)
     return cudaSuccess;
 }
 
+// Page-locked memory.  A submit may come while the caller captures a graph, also
+// in the modes that forbid allocation calls: these have no part in it.
+struct PageLocked {
+    static double *alloc(size_t bytes)
+    {
+        double *b = nullptr;
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+        const cudaError_t e = cudaHostAlloc((void **)&b, bytes, cudaHostAllocDefault);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (e == cudaSuccess) return b;
+        cudaGetLastError();
+        return nullptr;
+    }
+    static void free(double *b) { cudaFreeHost(b); }
+};
+
 #define TYPED_L(fn, L, prec, ...)                                                                   \
     ((prec) == LBM_FP64 ? fn<L, double>(__VA_ARGS__)                                                \
                         : (prec) == LBM_FP32 ? fn<L, float>(__VA_ARGS__)                            \
@@ -212,66 +229,14 @@ struct lbm_server {
     double gpu_ms = 0.0;
     int64_t rounds = 0;
     std::vector<Request *> retiring;     // results in flight
-    std::vector<std::pair<double *, size_t>> blocks;  // page-locked blocks kept for reuse
-    std::map<double *, size_t> held;     // blocks in use by requests
-    size_t kept = 0, held_bytes = 0;
-    size_t host_lend = size_t(1) << 30, host_keep = size_t(256) << 20;  // lbm_server_set_host_memory
+    // page-locked blocks of the requests' fields: a submitted request takes one
+    // while at most host_lend bytes are lent (lbm_server_set_host_memory)
+    HostBlocks<PageLocked> blocks{size_t(256) << 20};
+    size_t host_lend = size_t(1) << 30;
     std::string err;
 };
 
-// Page-locked host blocks.  Allocating and freeing one per request cost more
-// than its copies: the blocks of finished requests are kept for the next ones,
-// at most host_keep bytes of them, and given back when the server is
-// destroyed.  A submitted request takes one while requests hold at most
-// host_lend bytes of them.
 static size_t host_bytes(const Request *r) { return sizeof(double) * 4 * (size_t)r->ncell; }
-
-// A block of at least `bytes` (null: allocation failed)
-static double *take_block(lbm_server *s, size_t bytes)
-{
-    auto best = s->blocks.end();
-    for (auto it = s->blocks.begin(); it != s->blocks.end(); ++it)
-        if (it->second >= bytes && it->second <= 2 * bytes && (best == s->blocks.end() || it->second < best->second))
-            best = it;
-    double *b = nullptr;
-    size_t size = bytes;
-    if (best != s->blocks.end()) {
-        b = best->first;
-        size = best->second;
-        s->kept -= size;
-        s->blocks.erase(best);
-    } else {
-        // a submit may come while the caller captures a graph, also in the
-        // modes that forbid allocation calls: this one has no part in it
-        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
-        const cudaError_t e = cudaHostAlloc((void **)&b, bytes, cudaHostAllocDefault);
-        cudaThreadExchangeStreamCaptureMode(&mode);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-    }
-    s->held[b] = size;
-    s->held_bytes += size;
-    return b;
-}
-
-// Give a block back (its last use by the GPU has completed)
-static void return_block(lbm_server *s, double *b)
-{
-    if (!b) return;
-    auto it = s->held.find(b);
-    const size_t size = it->second;
-    s->held.erase(it);
-    s->held_bytes -= size;
-    if (s->kept + size > s->host_keep) {
-        cudaFreeHost(b);
-        return;
-    }
-    s->blocks.emplace_back(b, size);
-    s->kept += size;
-}
 
 static int sfail(lbm_server *s, int code, const char *fmt, ...)
 {
@@ -344,7 +309,7 @@ static void free_request_memory(lbm_server *s, Request *r)
 
 static void free_request_host(lbm_server *s, Request *r)
 {
-    return_block(s, r->host);
+    s->blocks.give(r->host);
     if (r->res_ev) cudaEventDestroy(r->res_ev);
     r->host = nullptr;
     r->res_ev = nullptr;
@@ -365,7 +330,6 @@ extern "C" void lbm_server_destroy(lbm_server_handle s)
         if (s->gpu_t0[k]) cudaEventDestroy(s->gpu_t0[k]);
         if (s->gpu_t1[k]) cudaEventDestroy(s->gpu_t1[k]);
     }
-    for (auto &b : s->blocks) cudaFreeHost(b.first);
     if (s->graph) cudaGraphExecDestroy(s->graph);
     for (int g = 0; g < NGROUPS; ++g) {
         if (s->tiles_d[g]) cudaFree(s->tiles_d[g]);
@@ -410,14 +374,14 @@ extern "C" int lbm_server_submit(lbm_server_handle s, const lbm_request *req, in
         return sfail(s, LBM_EINVAL, "request needs %zu bytes, more than the whole budget (%zu)", need, s->budget);
     }
     const size_t N = (size_t)r->ncell;
-    if (s->held_bytes + host_bytes(r) <= s->host_lend) r->host = take_block(s, host_bytes(r));
     try {
+        if (s->blocks.lent_bytes() + host_bytes(r) <= s->host_lend) r->host = s->blocks.take(host_bytes(r));
         if (!r->host) r->pageable.resize(4 * N);
         s->reqs[s->next_id] = r;
         s->queue.push_back(r);
     } catch (const std::bad_alloc &) {
         s->reqs.erase(s->next_id);
-        return_block(s, r->host);
+        s->blocks.give(r->host);
         delete r;
         return sfail(s, LBM_ENOMEM, "no host memory for a request of %zu cells", N);
     }
@@ -645,7 +609,7 @@ static int retire_slot(lbm_server *s, int k)
     cudaError_t e = cudaSuccess;
     if (r->aa && par) e = TYPED(unswap, r->lattice, r->prec, *r, s->doms_h[k].p, s->stream);
     if (e == cudaSuccess && !r->host) {
-        r->host = take_block(s, host_bytes(r));
+        r->host = s->blocks.take(host_bytes(r));
         if (!r->host) e = cudaErrorMemoryAllocation;
     }
     // the kernel writes the page-locked block over the host link
@@ -715,12 +679,7 @@ extern "C" int lbm_server_set_host_memory(lbm_server_handle s, size_t lend_bytes
 {
     if (!s) return sfail(nullptr, LBM_EINVAL, "null server");
     s->host_lend = lend_bytes;
-    s->host_keep = keep_bytes;
-    while (s->kept > s->host_keep) {
-        cudaFreeHost(s->blocks.front().first);
-        s->kept -= s->blocks.front().second;
-        s->blocks.erase(s->blocks.begin());
-    }
+    s->blocks.set_keep(keep_bytes);
     return LBM_OK;
 }
 
