@@ -11,11 +11,11 @@
 // at the warp's edge lanes).  Stores are aligned V-wide vectors of the
 // thread's own cells (the AA gather-push step stores its xi_x = +-1
 // populations one cell at a time).  Boundary roles are the ones of step.cuh:
-// rows on (or, for the AA steps, next to) a non-periodic y / z face take the
-// general update; a node on a non-periodic x face takes the streamed
-// populations of its x neighbour, which lives in the same thread, and its
-// velocity / pressure / free-slip role is applied to their moments in
-// registers.
+// rows that the vector path leaves (vec_row: 3D rows on a y / z face or whose
+// neighbours wrap, in-place rows next to a face) take the general update; a
+// node on a non-periodic x face takes the streamed populations of its x
+// neighbour, which lives in the same thread, and its velocity / pressure /
+// free-slip role is applied to their moments in registers.
 //
 // Reconstruction uses the parity of the Hermite terms: for an opposite pair
 // (i, i + Q/2) the even part E = a0 + H2:A2 / (2 c_s^4) is shared and the
@@ -301,25 +301,23 @@ __device__ __forceinline__ void gather_vec(const VecIn<L, S, C, V> &r, int k, C 
 }
 
 // Cell offsets from a row to the rows a pull reads: ym / yp for directions
-// with c_y > 0 / < 0 (the rows y - 1 / y + 1), zm / zp likewise in z.  WR = 0:
-// rows whose neighbours do not wrap (-nx, +nx, -nx ny, +nx ny); WR = 1: any
-// row of a lattice periodic in y and z, the neighbours of the first and last
-// rows wrapped around.  A push to the row y + c_y uses yp for c_y > 0 and ym
-// for c_y < 0.
+// with c_y > 0 / < 0 (the rows y - 1 / y + 1), zm / zp likewise in z.  2D: the
+// neighbours of the first and last rows wrapped around; 3D: rows whose
+// neighbours do not wrap (-nx, +nx, -nx ny, +nx ny).  A push to the row y + c_y
+// uses yp for c_y > 0 and ym for c_y < 0.
 struct RowOff {
     int ym, yp, zm, zp;
 };
 
-template <class L, int WR>
-__device__ __forceinline__ RowOff row_offsets(const StepParams &p, int y, int z)
+template <class L>
+__device__ __forceinline__ RowOff row_offsets(const StepParams &p, int y)
 {
-    const int nx = p.n[0], ny = p.n[1], nz = p.n[2], nxy = nx * ny;
+    const int nx = p.n[0], ny = p.n[1], nxy = nx * ny;
     RowOff o;
-    if (WR || L::D == 2) {
+    if (L::D == 2) {
         o.ym = y == 0 ? (ny - 1) * nx : -nx;
         o.yp = y == ny - 1 ? -(ny - 1) * nx : nx;
-        o.zm = L::D == 2 ? 0 : (z == 0 ? (nz - 1) * nxy : -nxy);
-        o.zp = L::D == 2 ? 0 : (z == nz - 1 ? -(nz - 1) * nxy : nxy);
+        o.zm = o.zp = 0;
     } else {
         o.ym = -nx;
         o.yp = nx;
@@ -494,7 +492,7 @@ __device__ __forceinline__ void add_shift(const StepParams &p, C *g, C sign)
 // non-periodic x face collides its neighbour's streamed populations: as they
 // are (outflow face) or with the face's density / velocity substituted; so do
 // the nodes of a row on the face row_inlet (>= 0, 2D).
-template <class L, class S, class C, int V, int G, int SP, int WR, bool SH>
+template <class L, class S, class C, int V, int G, int SP, bool SH>
 __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out0, int x0, int y, int z,
                                                   const RowOff &ro, const VecIn<L, S, C, V> &r, bool all_bulk,
                                                   int row_inlet)
@@ -552,7 +550,7 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
                 else
                     collide_fp64<L, true>(m, om, chi, o[kk]);
             } else {
-                rebuild_all<L, C, false, !WR>(cf, o[kk]);
+                rebuild_all<L, C, false, true>(cf, o[kk]);
             }
             add_shift<L, C, SH>(p, o[kk], C(-1));
         }
@@ -570,8 +568,8 @@ __device__ __forceinline__ void vec_collide_store(const StepParams &p, char *out
 // general update, V cells one after the other.  (Two rows, but they finish last.
 // GB300, us per step with / without the general update there: D2Q9 FP16
 // 1024 x 1024 periodic 7.96 / 6.95; between free-slip walls FP32 128 x 128
-// 2.70 / 1.93 (one cell per thread 1.86), 400 x 200 3.12 / 2.32 (2.43), 1024 x 1024
-// 8.88 / 8.08 (9.58).  The 3D kernels lost 2 % at 384 x 256 x 256 to the offsets that
+// 2.70 / 1.96 (one cell per thread 1.89), 400 x 200 3.12 / 2.31 (2.43), 1024 x 1024
+// 8.88 / 8.06 (9.67).  The 3D kernels lost 2 % at 384 x 256 x 256 to the offsets that
 // these rows need.)  The handle's sponge layers relax to the rest state (the
 // vector path's closed form) -- launch_update checks it.
 template <class L, int SP>
@@ -603,8 +601,9 @@ __device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z, int &
 // One thread's V cells of a row (x0 = first cell, a multiple of V); lanes
 // past the row end do nothing.  Rows outside the vector path update their
 // cells one by one with the general update (the same arithmetic).  in / out:
-// per-direction bases of the lattices (one lattice for the AA steps).  Used
-// by the single-lattice kernel and by the batched serving kernel.
+// per-direction bases of the lattices (one lattice for the AA steps).  (The
+// batched serving kernel has an update of its own, update_served, from the
+// same loads, collision and stores.)
 //
 // A node on a non-periodic x face takes the populations streamed into its
 // neighbour, which lives in the same thread; a velocity / free-slip /
@@ -615,29 +614,24 @@ __device__ __forceinline__ bool vec_row(const StepParams &p, int y, int z, int &
 // where it ran only for face cells, cost 13-17% of the whole kernel, and
 // updating the face cells in threads or a launch of their own (one cell per
 // row, so every access its own cache sector) cost more.
-//
-// WR = 1: a lattice periodic on every axis whose direction arrays span less
-// than 2 GB (32-bit offsets), as the serving engine's domains are: every row
-// takes the vector path, the first and last rows' neighbours wrapped
-// (row_offsets), and no general update is compiled in.
 // ---------------------------------------------------------------------------
-template <class L, class S, class C, int V, int G, int SP = kPull, int WR = 0, bool SH = false, bool CH = false>
+template <class L, class S, class C, int V, int G, int SP = kPull, bool SH = false, bool CH = false>
 __device__ __forceinline__ void update_vec(const StepParams &p, const char *const *in, char *const *out, int x0,
                                            int y, int z)
 {
     const int nx = p.n[0];
     if (x0 >= nx) return;  // lanes past the row end
     int sy = y, inlet = -1;
-    if (WR || vec_row<L, SP>(p, y, z, sy, inlet)) {
-        const RowOff ro = row_offsets<L, WR>(p, sy, z);
+    if (vec_row<L, SP>(p, y, z, sy, inlet)) {
+        const RowOff ro = row_offsets<L>(p, sy);
         VecIn<L, S, C, V> r;
         if (!vec_load<L, S, C, V, SP, CH>(p, in[0], x0, sy, z, ro, r)) return;
         const bool bulk = y >= p.blo[1] && y < p.bhi[1] && z >= p.blo[2] && z < p.bhi[2] && x0 >= p.blo[0] &&
                           x0 + V <= p.bhi[0];
-        vec_collide_store<L, S, C, V, G, SP, WR, SH>(p, out[0], x0, y, z, ro, r, bulk, L::D == 2 ? inlet : -1);
+        vec_collide_store<L, S, C, V, G, SP, SH>(p, out[0], x0, y, z, ro, r, bulk, L::D == 2 ? inlet : -1);
         return;
     }
-    if constexpr (!WR) {
+    if constexpr (L::D == 3 || SP != kPull) {  // (the 2D pull leaves no row)
 #pragma unroll 1
         for (int k = 0; k < V; ++k) {
             if (SP == kPull)
@@ -674,7 +668,7 @@ template <class L, class S, class C, int V, int SP, bool SH = false, bool CH = f
 __global__ void __launch_bounds__(256, (VecMinBlocks<L, S, V, SP>::value)) k_stream_collide_vec(const __grid_constant__ StepParams p)
 {
     if constexpr (CH) chain_begin(p);
-    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, 0, SH, CH>(
+    update_vec<L, S, C, V, VecGroup<S, V>::value, SP, SH, CH>(
         p, p.in, p.out, (blockIdx.x * blockDim.x + threadIdx.x) * V, sweep_y(p), sweep_z(p));
 }
 
