@@ -79,8 +79,9 @@ inline int vec_default(int lattice, int precision)
 // update, in the vectorised kernel V cells one after the other, and finish last.
 // GB300, us per step, one cell / two (inlet, outflow on the other faces): FP32
 // 128^2 4.12 / 5.57, 512^2 6.87 / 7.38, 700 x 400 7.19 / 7.69, 1024 x 512 9.95 / 9.14;
-// FP16 128^2 4.23 / 5.38, 256^2 4.55 / 5.64, 512^2 7.09 / 6.77.
-inline bool aa_small_2d(int64_t ncell, size_t elem) { return ncell <= (int64_t)elem << 16; }
+// FP16 128^2 4.23 / 5.38, 256^2 4.55 / 5.64, 512^2 7.09 / 6.77.  The lines through these
+// cross at 360 000 and 210 000 cells.
+inline bool aa_small_2d(int64_t ncell, size_t elem) { return ncell <= (elem == 4 ? 360000 : 210000); }
 // Default threads per block.  The vectorised kernel's blocks lie along x
 // rows of nx / vec threads, so the block has to divide the row's warps or the
 // last block of every row holds idle warps: 64 threads where the row is a

@@ -91,8 +91,8 @@ def test_default_shape_between_walls_is_not_the_slower_one(prec, n):
     assert step_us(n, prec, kinds, False, 0) < 1.25 * step_us(n, prec, kinds, False, 1)
 
 
-@pytest.mark.parametrize("prec,n,cells", [("fp32", (512, 512, 1), 1), ("fp32", (512, 514, 1), 2), ("fp16", (512, 256, 1), 1),
-                                          ("bf16", (512, 258, 1), 2), ("fp32", (64, 6, 1), 1)])
+@pytest.mark.parametrize("prec,n,cells", [("fp32", (600, 600, 1), 1), ("fp32", (600, 602, 1), 2), ("fp16", (600, 350, 1), 1),
+                                          ("bf16", (600, 352, 1), 2), ("fp32", (64, 6, 1), 1)])
 @pytest.mark.parametrize("walls", [True, False])
 def test_small_in_place_lattices_take_one_cell_per_thread(prec, n, cells, walls):
     """At the edges of the rule; a periodic y axis keeps two, as does the pull."""
