@@ -307,9 +307,14 @@ int lbm_probe(lbm_handle h, int n, const int64_t *cells, double *p_prime);
  * is configured now, complete or not.  An explicitly set shape is reported as
  * set also under plain BGK, order 4 and sponges that the vectorised kernel does
  * not take, where the general kernel runs instead.
+ *
+ * lbm_get_sweep reports whether the next step takes the rows of level 0 from
+ * the last to the first: every other step does where a step moves more than
+ * twice the bytes of the L2 cache (the result does not depend on it).
  */
 int lbm_set_launch(lbm_handle h, int block, int cells_per_thread);
 int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread);
+int lbm_get_sweep(lbm_handle h, int *backwards);
 
 /*
  * lbm_pressure_mean / lbm_pressure_fluctuation -- the fluctuating pressure

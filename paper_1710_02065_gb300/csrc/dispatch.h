@@ -97,6 +97,17 @@ inline int block_default(int vec, int nx)
     return row % 64 == 0 ? 64 : (row <= 96 ? row : 32);
 }
 
+// Every other step (odd) sweeps the lattice backwards (sweep_y) where a step
+// moves over twice the L2's bytes.  GB300, us per pass, forwards / alternating:
+// D3Q27 FP16 192 x 128 x 128 jet (340 MB a step) 5011 / 4871, D3Q19 384 x 256 x 256 jets
+// FP16 (1.9 GB) 18236 / 18131, BF16 in place 21825 / 21548; below, the rows are in L2
+// either way and it gained nothing (D3Q19 FP16 161 x 129 x 97, 150 MB, 4075 / 4117;
+// D2Q9 FP16 1024^2 1619 / 1634).
+inline bool sweep_back(int q, size_t elem, int64_t ncell, int64_t l2_bytes, bool odd)
+{
+    return odd && 2 * (int64_t)elem * q * ncell > 2 * l2_bytes;
+}
+
 // Row-staged kernel (bulk copies of whole rows into shared memory; FP32,
 // FP16, BF16; no cell-type mask; nx * element size a multiple of 16 bytes).
 struct RowsPlan {

@@ -1405,6 +1405,14 @@ static cudaError_t ensure_side_stream(lbm_ctx *h)
 
 static cudaError_t advance_level(lbm_ctx *h, std::vector<StepParams> &params, int k, int64_t step);
 
+// Whether the next step of a level sweeps it backwards
+static int level_back(lbm_ctx *h, int k)
+{
+    const GridRef g = level_grid(h, k);
+    const bool aa = k == 0 && h->pattern == LBM_STREAM_AA;
+    return sweep_back(h->q, h->elem, g.ncell, h->l2_bytes, (aa ? h->aa_odd : *g.cur) != 0) ? 1 : 0;
+}
+
 // The child's part of a step of level k: two steps of level k + 1 with its
 // ring refilled at t + 1/2 and t + 1, and the covered ring of level k rebuilt
 // from the child at t + 1/2.
@@ -1431,18 +1439,6 @@ static cudaError_t advance_child(lbm_ctx *h, std::vector<StepParams> &params, in
 // with the level-0 update, which is HBM-bound while the child's interface
 // kernels are latency-bound; the level-0 stream waits for it before the next
 // step.  The result is bitwise that of running the two in order.
-//
-// Every other step sweeps the lattice backwards (sweep_y) where a step moves
-// over twice the L2's bytes.  GB300, us per pass, forwards / alternating: D3Q27
-// FP16 192 x 128 x 128 jet (340 MB a step) 5011 / 4871, D3Q19 384 x 256 x 256 jets
-// FP16 (1.9 GB) 18236 / 18131, BF16 in place 21825 / 21548; below, the rows are in
-// L2 either way and it gained nothing (D3Q19 FP16 161 x 129 x 97, 150 MB, 4075 /
-// 4117; D2Q9 FP16 1024^2 1619 / 1634).
-static int sweep_back(const lbm_ctx *h, int64_t ncell, int odd)
-{
-    return 2 * h->q * ncell * (int64_t)h->elem > 2 * (int64_t)h->l2_bytes ? odd : 0;
-}
-
 static cudaError_t advance_level(lbm_ctx *h, std::vector<StepParams> &params, int k, int64_t step)
 {
     const bool child = k < (int)h->levels.size();
@@ -1451,7 +1447,7 @@ static cudaError_t advance_level(lbm_ctx *h, std::vector<StepParams> &params, in
     GridRef g = level_grid(h, k);
     params[k].step = step;
     const bool aa = k == 0 && h->pattern == LBM_STREAM_AA;  // (never with refined levels)
-    params[k].back = sweep_back(h, g.ncell, aa ? h->aa_odd : *g.cur);
+    params[k].back = level_back(h, k);
     if (e == cudaSuccess && child && k == 0 && h->level_overlap && !aa) {
         const void *fin = g.f[*g.cur];
         void *fout = g.f[1 - *g.cur];
@@ -1830,6 +1826,13 @@ extern "C" int lbm_get_launch(lbm_handle h, int *block, int *cells_per_thread)
     const int vec = pick_vec(h, p);
     if (block) *block = h->block > 0 ? h->block : block_default(vec, h->n[0]);  // level 0
     if (cells_per_thread) *cells_per_thread = vec;
+    return LBM_OK;
+}
+
+extern "C" int lbm_get_sweep(lbm_handle h, int *backwards)
+{
+    CHECK_HANDLE(h);
+    if (backwards) *backwards = level_back(h, 0);
     return LBM_OK;
 }
 

@@ -70,6 +70,7 @@ _sig("lbm_reduce", [_h, _dp, _dp])
 _sig("lbm_probe", [_h, C.c_int, _i64p, _dp])
 _sig("lbm_sync", [_h])
 _sig("lbm_set_launch", [_h, C.c_int, C.c_int])
+_sig("lbm_get_sweep", [_h, _ip])
 _sig("lbm_get_launch", [_h, _ip, _ip])
 _sig("lbm_set_staging", [_h, C.c_int, C.c_int, C.c_int])
 _sig("lbm_set_transfer_staging", [_h, C.c_size_t])
@@ -298,6 +299,12 @@ def lbm_get_launch(h):
 
 
 LBM_COLLISION_RR, LBM_COLLISION_BGK = 0, 1
+
+
+def lbm_get_sweep(h) -> bool:
+    b = C.c_int()
+    _check(_lib.lbm_get_sweep(h, C.byref(b)), h)
+    return b.value != 0
 
 
 def lbm_set_sponge_jet_reference(h, yc: float, zc: float, U_jet: float, D: float, x0: float, B: float = 5.8,
