@@ -580,13 +580,16 @@ static cudaError_t enqueue_steps(lbm_server *s, int64_t steps)
     return cudaGetLastError();
 }
 
-// Streams and events of the chains the next round needs (before its capture)
+// Streams and events of the chains the next round needs (before its capture);
+// the streams have the priority of the server's
 static cudaError_t ensure_chains(lbm_server *s)
 {
     cudaError_t e = s->fork_ev ? cudaSuccess : cudaEventCreateWithFlags(&s->fork_ev, cudaEventDisableTiming);
+    int priority = 0;
+    if (e == cudaSuccess) e = cudaStreamGetPriority(s->stream, &priority);
     for (int g = 0; g < NGROUPS && e == cudaSuccess; ++g) {
         if (s->tiles_h[g].empty() || s->side[g]) continue;
-        e = cudaStreamCreateWithFlags(&s->side[g], cudaStreamNonBlocking);
+        e = cudaStreamCreateWithPriority(&s->side[g], cudaStreamNonBlocking, priority);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->join_ev[g], cudaEventDisableTiming);
     }
     return e;
