@@ -718,8 +718,8 @@ def run_serving(lbm, torch, args):
                            "bytes": "2 Q s per cell update of every request, over the device time of the rounds"}
     out["arrival_rate_note"] = ("default rate 9.7/s: 0.8 x the 12.1 requests/s this stream was served at when "
                                 "saturated by the first engine (35.0 G cell updates/s), kept for comparison; the "
-                                "current engine serves it at 13.8 requests/s saturated (1.48e12 cell updates at "
-                                "39.9 G/s with arrivals at 40/s), so 9.7/s is 0.70 x saturation")
+                                "current engine serves it at 17.8 requests/s saturated (1.48e12 cell updates at "
+                                "51.7 G/s with arrivals at 40/s), so 9.7/s is 0.54 x saturation")
     return out
 
 
@@ -827,8 +827,8 @@ def main():
     ap.add_argument("--cyl-steps", type=int, default=40000, help="fine-resolution steps of the cylinder runs")
     ap.add_argument("--requests", type=int, default=512)
     ap.add_argument("--rate", type=float, default=9.7,
-                    help="serving arrival rate (requests/s); the default 9.7/s is 0.70 x the 13.8 requests/s "
-                         "this stream is served at when saturated (1.48e12 cell updates at 39.9 G/s)")
+                    help="serving arrival rate (requests/s); the default 9.7/s is 0.54 x the 17.8 requests/s "
+                         "this stream is served at when saturated (1.48e12 cell updates at 51.7 G/s)")
     ap.add_argument("--steps-scale", type=float, default=1.0, help="serving: scale of per-request steps")
     ap.add_argument("--budget-gb", type=float, default=8.0, help="serving: HBM budget for populations")
     ap.add_argument("--round-steps", type=int, default=100, help="serving: steps per batched round")
