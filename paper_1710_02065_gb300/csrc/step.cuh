@@ -564,15 +564,20 @@ __device__ __forceinline__ void cell_collide(const StepParams &p, const Mom<C> &
 // The loads of 3D 16-bit storage only in rows without x faces: a warp at an x
 // sponge runs both forms (161 x 129 x 97 open box, us per step with / without:
 // D3Q19 FP16 39.9 / 39.1, D3Q27 FP16 56.7 / 55.1; 95 x 64 x 64 D3Q27 FP16 13.0 / 12.4).
-template <class L, class S>
+// Nor in 16-bit updates whose other code crowds it out: next to solids (D2Q9 FP16
+// 401 x 203 cylinder 3.77 / 3.44, D3Q27 FP16 96 x 64 x 64 13.9 / 13.5), in 3D beside
+// refined levels (D3Q19 FP16 128 x 96 x 96 116.0 / 114.0) and in plain BGK on D3Q19
+// (64 registers instead of 48: FP16 128^3 40.6 / 33.8).
+template <class L, class S, bool BGK, int MASK>
 __host__ __device__ constexpr bool uniform_rows()
 {
-    return L::D == 2 || sizeof(S) != 4;
+    if (sizeof(S) == 2) return !(BGK && L::Q == 19) && (L::D == 2 ? MASK != kMaskLinks : MASK == kMaskNone);
+    return L::D == 2 || sizeof(S) == 8;
 }
-template <class L, class S>
+template <class L, class S, bool BGK, int MASK>
 __device__ __forceinline__ bool uniform_loads(const StepParams &p)
 {
-    return uniform_rows<L, S>() && p.off32 && (L::D == 2 || sizeof(S) == 8 || p.periodic[0]);
+    return uniform_rows<L, S, BGK, MASK>() && p.off32 && (L::D == 2 || sizeof(S) == 8 || p.periodic[0]);
 }
 
 template <class L, class S, class C, bool BGK = false, int MASK = kMaskLinks, bool CH = false>
@@ -646,7 +651,7 @@ __device__ __forceinline__ void update_cell(const StepParams &p, const char *con
             if (p.shifted) g[i] += dsh<C>(p, k);
         }
     } else {
-        if (uniform_loads<L, S>(p) && bulk && (unsigned)(y - 1) < ny - 2 && (L::D == 2 || (unsigned)(z - 1) < nz - 2)) {
+        if (uniform_loads<L, S, BGK, MASK>(p) && bulk && (unsigned)(y - 1) < ny - 2 && (L::D == 2 || (unsigned)(z - 1) < nz - 2)) {
             // rows that do not wrap: each direction's row is a fixed distance from
             // the cell's, the same for every thread, so the addresses are three
             // 32-bit offsets (x, x - 1, x + 1) on uniform bases
@@ -682,7 +687,7 @@ __device__ __forceinline__ void update_cell(const StepParams &p, const char *con
     }
     // (the stores likewise: two-level cylinder 1485 -> 1472 us, D3Q19 FP16 161 x 129 x 97
     // box 4083 -> 4011; D3Q27 FP16 jet 4746 -> 4884, so not there)
-    if (uniform_rows<L, S>() && L::Q <= 19 && p.off32) {
+    if (uniform_rows<L, S, BGK, MASK>() && L::Q <= 19 && p.off32) {
 #pragma unroll
         for (int i = 0; i < L::Q; ++i) Store<S>::st((S *)(out[i] + cell * (unsigned)sizeof(S)), o[i]);
     } else {
