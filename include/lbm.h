@@ -644,7 +644,8 @@ int lbm_load(lbm_handle h, const char *path);
  *   lbm_server_gpu_time : device time of all rounds' graphs so far (ms, CUDA
  *                       events around each replay; waits for the stream)
  * Errors: LBM_EINVAL (bad request, a request larger than the whole budget,
- * unknown id, result of an unfinished request), LBM_ECUDA.
+ * unknown id, result of an unfinished request), LBM_ENOMEM (no host memory for a
+ * request's fields; nothing is queued), LBM_ECUDA.
  */
 typedef struct lbm_server *lbm_server_handle;
 
